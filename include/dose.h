@@ -150,28 +150,33 @@ typedef struct {
              (default);
          1 = CSR (per-row scatter; the row-group layout is not built);
          2 = row groups (create fails with DOSE_ERR_UNSUPPORTED if they do not apply).
-       Row groups: up to four consecutive non-empty rows share one list of the union of
-       their columns, with the four rows' values stored side by side (stored zeros where
-       a row has no entry); built when no row has more than 4096 entries.  The union
-       order is chosen per group (shared-memory banks), so these passes sum a row's terms
-       in another order than dose_spmv.  A non-finite x_j or residual reaches every row
-       of a group whose union holds column j (0 * inf), not only the rows that store j. */
+       Row groups: up to eight rows (four where that stores less, and for F32) that see
+       nearly the same columns share one list of the union of their columns, with the
+       rows' values stored side by side (stored zeros where a row has no entry); built
+       when no row has more than 4096 entries.  The rows of a group need not be
+       consecutive: on a voxel grid, whose strides are looked for in the matrix, they are
+       neighbours along the beam or small cubes.  The union order is chosen per group
+       (shared-memory banks), so these passes sum a row's terms in another order than the
+       CSR forms.  A non-finite x_j or residual reaches every row of a group whose union
+       holds column j (0 * inf), not only the rows that store j. */
     uint32_t adj_layout;
-    uint32_t rg_tile_union;     /* row groups: union columns per pipeline stage (512..8192; default
-                                   by format, about 24 KB of columns and values) */
-    uint32_t rg_tile_rows;      /* row groups: rows per stage (256..8192) */
-    uint32_t rg_stages;         /* row groups: pipeline depth (2..8) */
-    uint32_t rg_warps;          /* row groups: worker warps (1..15; 0 = as many as fit) */
-    uint32_t rg_l2_prefetch;    /* row groups: stages prefetched into L2 ahead of the ring (1..31;
-                                   0 = default, off; 32 = off) */
+    uint32_t rg_tile_union;     /* row groups: most union columns per packet (what one warp copies at a
+                                   time; 256..8192, at most 320 are used; default 320).  Packets are cut
+                                   at create; a later value is checked and reported only.  It must not
+                                   be smaller than the longest row. */
+    uint32_t rg_tile_rows;      /* row groups: checked and reported (256..8192); a packet holds at most 64 rows */
+    uint32_t rg_stages;         /* row groups: packets in flight per warp of the adjoint and fused passes
+                                   (2..8; at most 4 are used; default 2) */
+    uint32_t rg_warps;          /* row groups: worker warps of those passes (1..15; 0 = as many as fit) */
+    uint32_t rg_l2_prefetch;    /* row groups: checked and reported; the passes need no L2 prefetch */
     uint32_t fwd_layout;        /* layout dose_spmv runs on: 0 = row groups where the handle has them
                                    (and not DOSE_CREATE_COMPENSATED, whose long-row sums run on CSR),
                                    else CSR (default); 1 = CSR; 2 = row groups (create and
                                    dose_set_tuning fail if dose_spmv cannot take them).  On row groups
                                    a row's terms are added in its group's union order (see adj_layout),
-                                   so the last bits may differ from the CSR form's.  dose_spmv_f64
-                                   takes the row-group form only with fwd_layout = 2 (its arithmetic,
-                                   not its bytes, bounds it, and CSR is faster for it). */
+                                   so the last bits may differ from the CSR form's.  dose_spmv_f64 follows
+                                   dose_spmv, except that DOSE_SPMV_F64_NATIVE takes row groups only with
+                                   fwd_layout = 2 (FP64 FMAs bound it, and CSR stores fewer values). */
 } dose_tuning;
 
 typedef struct {
@@ -202,8 +207,8 @@ typedef struct {
     uint32_t adj_layout_fused;  /* layout the fused pass runs on: 1 = CSR, 2 = row groups, 0 = none fits */
     uint32_t adj_layout_adjoint;/* ... dose_adjoint */
     uint64_t rg_groups;         /* row groups built (0: the layout was not built) */
-    uint64_t rg_union_entries;  /* union columns of all groups (values stored: 4 per union column) */
-    uint32_t rg_window;         /* columns of each CTA's gradient window on the row-group layout */
+    uint64_t rg_union_entries;  /* values stored by the row groups / 4 (union columns x rows per group / 4) */
+    uint32_t rg_window;         /* most columns any CTA sees on the row-group layout */
     uint32_t rg_warps_fused;    /* worker warps of the row-group fused pass (0 if it does not fit) */
     uint32_t rg_index_bytes;    /* bytes per union column index (2 when ncols <= 65536, else 4) */
     uint32_t rg_pad;

@@ -538,21 +538,17 @@ dose_status sweep(dose_matrix* A, const float* x, unsigned purposes, cudaStream_
         const bool time_v = (purposes & DOSE_TUNE_FORWARD) && !(A->flags & DOSE_CREATE_SELL) && A->rg.built &&
                             A->fwd.tuning.layout != 1;
         const AdjTuning base = A->adj_tuning;
-        AdjTuning rg_cut = base, csr_cut = base;  // knobs the two adjoint schedules are cut with
+        AdjTuning csr_cut = base;  // knobs the CSR adjoint schedule is cut with
         std::vector<AdjTuning> cands{base};
         if (A->rg.built) {
-            for (uint32_t tu : {0u, 2048u, 3072u, 4096u, 6144u})
-                for (uint32_t tr : {512u, 1024u})
-                    for (uint32_t wn : {0u, 12u})
-                        for (uint32_t sd : {2u, 3u}) {
-                            AdjTuning a = base;
-                            a.layout = 0;
-                            a.rg_tile_u = tu;
-                            a.rg_tile_rows = tr;
-                            a.rg_warps = wn;
-                            a.rg_stages = sd;
-                            cands.push_back(a);
-                        }
+            for (uint32_t wn : {0u, 12u, 10u, 8u})
+                for (uint32_t sd : {2u, 3u, 4u}) {
+                    AdjTuning a = base;
+                    a.layout = 0;
+                    a.rg_warps = wn;
+                    a.rg_stages = sd;
+                    cands.push_back(a);
+                }
             AdjTuning a = base;
             a.layout = 1;  // the CSR layout, for comparison
             cands.push_back(a);
@@ -567,23 +563,13 @@ dose_status sweep(dose_matrix* A, const float* x, unsigned purposes, cudaStream_
                         cands.push_back(a);
                     }
         }
-        // Re-cut what a candidate changes; *usable = false when its stage cannot
-        // hold a group's union (the previous cut is then restored).
+        // Re-cut (CSR) or deal anew (row groups) what a candidate changes; *usable =
+        // false where its knobs are out of range.
         auto cut = [&](const AdjTuning& a, bool* usable) -> dose_status {
             *usable = true;
             if (check_adj_tuning(a) != DOSE_OK) {
                 *usable = false;
                 return DOSE_OK;
-            }
-            if (A->rg.built && (a.rg_tile_u != rg_cut.rg_tile_u || a.rg_tile_rows != rg_cut.rg_tile_rows)) {
-                cudaError_t e2 = rg_schedule(A, a);
-                if (e2 == cudaErrorInvalidValue) {
-                    *usable = false;
-                    e2 = rg_schedule(A, rg_cut);
-                }
-                if (e2 != cudaSuccess) return cuda_fail(e2, "row-group schedule");
-                if (!*usable) return DOSE_OK;
-                rg_cut = a;
             }
             if (a.tile_nnz != csr_cut.tile_nnz || a.tile_rows != csr_cut.tile_rows || a.stages != csr_cut.stages ||
                 a.row_order != csr_cut.row_order) {
@@ -592,6 +578,10 @@ dose_status sweep(dose_matrix* A, const float* x, unsigned purposes, cudaStream_
                 csr_cut = a;
             }
             A->adj_tuning = a;
+            if (A->rg.built) {
+                const cudaError_t e2 = rg_schedule(A);
+                if (e2 != cudaSuccess) return cuda_fail(e2, "row-group schedule");
+            }
             return DOSE_OK;
         };
         float best = 3e38f;

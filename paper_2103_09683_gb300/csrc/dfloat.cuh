@@ -34,6 +34,17 @@ __device__ __forceinline__ void df_add(float& s, float& c, float s2, float c2) {
     c = __fadd_rn(c, __fadd_rn(c2, e));
 }
 
+// x_j as the kernels hold it: the FP32 pair (hi, lo), or the double itself.
+template <int MODE>
+__device__ __forceinline__ uint2 prepare_x(double v) {
+    if (MODE == F64_DF) {
+        const float hi = __double2float_rn(v);
+        const float lo = __double2float_rn(v - (double)hi);  // v - hi is exact in FP64
+        return make_uint2(__float_as_uint(hi), __float_as_uint(lo));
+    }
+    return make_uint2((uint32_t)__double2loint(v), (uint32_t)__double2hiint(v));
+}
+
 // Accumulator of one lane: a double-float pair or a double.
 template <int MODE>
 struct Acc;

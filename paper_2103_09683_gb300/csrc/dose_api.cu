@@ -382,7 +382,8 @@ static void free_dev_schedule(DevSchedule& D) {
 }
 
 static void free_all(dose_matrix* A) {
-    free_row_groups(A);
+    free_row_groups(A->rg);
+    free_row_groups(A->rgf);
     free_dev_schedule(A->fwd);
     free_dev_schedule(A->fwd64);
     free_dev_schedule(A->adj);
@@ -624,9 +625,11 @@ dose_status dose_encode_host(dose_format fmt, uint32_t nrows, const uint32_t* ro
     return encode(fmt, nrows, row_ptr, nnz, values_f64, codes, scales);
 }
 
-dose_status dose_create_matrix(const dose_csr_desc* desc, unsigned flags, const dose_tuning* tuning, void* stream,
-                               dose_matrix** out) {
-    NvtxRange nvtx_range("dose_create_matrix");
+}  // extern "C"
+
+// plan: the merged matrix of several beams (dose_create_multibeam).
+static dose_status create_matrix(const dose_csr_desc* desc, unsigned flags, const dose_tuning* tuning, void* stream,
+                                 bool plan, dose_matrix** out) {
     if (!desc || !out) return invalid("dose_create_matrix: null desc or out");
     *out = nullptr;
     if (flags & ~(DOSE_CREATE_COMPENSATED | DOSE_CREATE_U16_INDEX | DOSE_CREATE_SELL))
@@ -862,9 +865,22 @@ dose_status dose_create_matrix(const dose_csr_desc* desc, unsigned flags, const 
     // Row-group layout of the adjoint and fused passes (unless the caller asked for CSR).
     if (A->adj_tuning.layout != 1) {
         std::string why;
-        A->rg.sched.grid = A->adj.grid;
-        bool ok = build_row_groups(A.get(), A->host_row_ptr.data(), col.data(), vals.data(), &why, &e);
-        if (!ok && e != cudaSuccess) {
+        A->rg.grid = A->rgf.grid = A->adj.grid;
+        bool ok = build_row_groups(A.get(), A->rg, false, A->host_row_ptr.data(), col.data(), vals.data(), scl.data(), &why, &e);
+        uint64_t full = 0;
+        for (uint32_t i = 0; i < nrows; ++i) full += A->host_row_ptr[i + 1] > A->host_row_ptr[i];
+        if (ok && (plan || full < kRgKeepRows) &&
+            !build_row_groups(A.get(), A->rgf, true, A->host_row_ptr.data(), col.data(), vals.data(), scl.data(), &why, &e)) {
+            free_row_groups(A->rg);
+            ok = false;
+        }
+        if (!ok && e == cudaErrorInvalidValue) {
+            why = "tuning.rg_tile_union is smaller than the longest row";
+            if (A->adj_tuning.layout == 2) {
+                free_all(A.get());
+                return invalid(why);
+            }
+        } else if (!ok && e != cudaSuccess) {
             // the layout is optional by default: without the memory for it the
             // handle keeps the CSR passes (asked for explicitly, it is an error)
             if (e != cudaErrorMemoryAllocation || A->adj_tuning.layout == 2) return fail(e, "row-group layout");
@@ -872,19 +888,12 @@ dose_status dose_create_matrix(const dose_csr_desc* desc, unsigned flags, const 
             why = "its arrays do not fit in device memory";
         }
         if (ok) {
-            e = rg_schedule(A.get(), A->adj_tuning);
+            e = rg_schedule(A.get());
             if (e == cudaErrorMemoryAllocation && A->adj_tuning.layout != 2) {
                 cudaGetLastError();
-                free_row_groups(A.get());
+                free_row_groups(A->rg);
+                free_row_groups(A->rgf);
                 ok = false;
-            } else if (e == cudaErrorInvalidValue) {
-                why = "tuning.rg_tile_union is smaller than a group's union of columns";
-                free_row_groups(A.get());
-                ok = false;
-                if (A->adj_tuning.layout == 2) {
-                    free_all(A.get());
-                    return invalid(why);
-                }
             } else if (e != cudaSuccess) {
                 return fail(e, "row-group schedule");
             }
@@ -901,7 +910,7 @@ dose_status dose_create_matrix(const dose_csr_desc* desc, unsigned flags, const 
                   std::string((flags & DOSE_CREATE_COMPENSATED) ? " (DOSE_CREATE_COMPENSATED sums on CSR)" : ""));
         return DOSE_ERR_UNSUPPORTED;
     }
-    A->device_bytes = A->rg.bytes + (A->rg.built ? (A->rg.host.size() + 1) * 16 + schedule_bytes(A->rg.sched) : 0) +
+    A->device_bytes = A->rg.bytes + A->rgf.bytes +
                       A->sell.bytes + rp_alloc * 4 + col_alloc * 4 + ((flags & DOSE_CREATE_U16_INDEX) ? col16_alloc * 2 : 0) + val_alloc +
                       (fmt == DOSE_FMT_FP8E4M3_ROWSCALE ? ((size_t)nrows + 16) * 4 : 0) + x64_alloc * 8 +
                       (size_t)A->adj.grid * ncols_pad * 4 + (size_t)A->adj.grid * 8 + 4 + schedule_bytes(A->fwd) +
@@ -923,6 +932,14 @@ dose_status dose_create_matrix(const dose_csr_desc* desc, unsigned flags, const 
     }
     *out = H;
     return DOSE_OK;
+}
+
+extern "C" {
+
+dose_status dose_create_matrix(const dose_csr_desc* desc, unsigned flags, const dose_tuning* tuning, void* stream,
+                               dose_matrix** out) {
+    NvtxRange nvtx_range("dose_create_matrix");
+    return create_matrix(desc, flags, tuning, stream, false, out);
 }
 
 dose_status dose_create_multibeam(const dose_csr_desc* beams, int nbeams, unsigned flags, const dose_tuning* tuning,
@@ -996,7 +1013,7 @@ dose_status dose_create_multibeam(const dose_csr_desc* beams, int nbeams, unsign
         m.values = val.data();
         m.scales = b0.scales;
     }
-    return dose_create_matrix(&m, flags, tuning, stream, out);
+    return create_matrix(&m, flags, tuning, stream, true, out);
 }
 
 dose_status dose_destroy(dose_matrix* A) {
@@ -1037,7 +1054,7 @@ namespace dose {
 // (fwd_layout = 1), the handle sums long rows with compensation (a CSR path),
 // or the layout is missing or its ring does not fit beside the window of x.
 bool spmv_on_row_groups(const dose_matrix* A) {
-    return A->fwd.tuning.layout != 1 && !(A->flags & DOSE_CREATE_COMPENSATED) && rg_spmv_applies(A, nullptr, nullptr);
+    return A->fwd.tuning.layout != 1 && !(A->flags & DOSE_CREATE_COMPENSATED) && rg_forward_warps(A, RG_DEAL_SPMV, nullptr, nullptr) > 0;
 }
 
 dose_status adjoint_supported(const dose_matrix* A, bool quad, const float* const* vecs, int nvec) {
@@ -1185,21 +1202,20 @@ dose_status dose_matrix_info(const dose_matrix* A, dose_info* out) {
     out->adj_layout_fused = out->adj_block_fused ? 1 : 0;
     out->adj_layout_adjoint = out->adj_block_adjoint ? 1 : 0;
     if (A->rg.built) {
-        out->rg_groups = A->rg.host.size();
-        out->rg_union_entries = A->rg.n_union;
-        out->rg_window = A->rg.sched.wwidth;
+        out->rg_groups = A->rg.n_groups;
+        out->rg_union_entries = A->rg.n_union * A->rg.hr / 4;
+        out->rg_window = A->rg.wmax;
         out->rg_index_bytes = A->rg.iw;
-        out->tuning.rg_tile_union = A->rg.tile_u;
-        size_t smem = 0;
-        out->rg_warps_fused = rg_shape(A, A->adj_tuning, true, &smem);
+        out->tuning.rg_tile_union = A->adj_tuning.rg_tile_u ? A->adj_tuning.rg_tile_u : A->rg.tile_u;
+        out->rg_warps_fused = rg_gradient_warps(A, A->adj_tuning, true, nullptr, nullptr);
         if (rg_active(A, true)) {
             out->adj_layout_fused = 2;
-            out->adj_block_fused = 32 * (1 + out->rg_warps_fused);
+            out->adj_block_fused = 32 * out->rg_warps_fused;
             out->fused_bytes = rg_fused_bytes(A, false);
         }
         if (rg_active(A, false)) {
             out->adj_layout_adjoint = 2;
-            out->adj_block_adjoint = 32 * (1 + rg_shape(A, A->adj_tuning, false, &smem));
+            out->adj_block_adjoint = 32 * rg_gradient_warps(A, A->adj_tuning, false, nullptr, nullptr);
             out->adjoint_bytes = rg_adjoint_bytes(A);
         }
     }
@@ -1223,17 +1239,10 @@ dose_status dose_set_tuning(dose_matrix* A, const dose_tuning* tuning) {
     if (at.layout == 2 && !A->rg.built) return invalid("adj_layout = 2: the handle has no row-group layout");
     if (t.layout == 2 && (!A->rg.built || (A->flags & DOSE_CREATE_COMPENSATED)))
         return invalid("fwd_layout = 2: dose_spmv cannot run on the row-group layout of this handle");
-    const AdjTuning old_at = A->adj_tuning;
+    if (A->rg.built && at.rg_tile_u != A->adj_tuning.rg_tile_u && A->max_row_len > at.rg_tile_u)
+        return invalid("tuning.rg_tile_union is smaller than the longest row");
     A->adj_tuning = at;
-    if (A->rg.built && (at.rg_tile_u != old_at.rg_tile_u || at.rg_tile_rows != old_at.rg_tile_rows)) {
-        e = rg_schedule(A, at);
-        if (e == cudaErrorInvalidValue) {
-            A->adj_tuning = old_at;
-            rg_schedule(A, old_at);
-            return invalid("tuning.rg_tile_union is smaller than a group's union of columns");
-        }
-        if (e != cudaSuccess) return cuda_fail(e, "row-group schedule");
-    }
+    if (A->rg.built && (e = rg_schedule(A)) != cudaSuccess) return cuda_fail(e, "row-group schedule");
     return apply_schedule(A, A->adj, adj_schedule_tuning(t, at), true);
 }
 

@@ -116,40 +116,86 @@ struct DealItem {
     uint64_t cost;
 };
 
-// Row-group layout of a matrix, built at create for the adjoint and the fused
-// objective pass.  The non-empty rows, in matrix order, are cut into groups of
-// up to four consecutive ones whose columns mostly coincide (neighbouring voxels
-// see the same spots).  A group stores the union of its rows' columns once and,
-// for each union column, the four rows' stored values side by side (the stored
-// zero where a row has no entry).  One warp then takes a whole group: per union
-// column one gather of x feeds four rows' dot products, and after the four
-// residuals are known one read-modify-write of the gradient accumulator adds
-// all four rows' contributions.
-//   stage (StageDesc reused): rows [row0, row1), union entries [nz0, nz1),
-//   groups [ne0, ne1); meta unused.
-//   group record (uint4): x = first union entry, y = union size, z / w = the
-//   rows' offsets from the stage's row0 as u16 pairs (0xFFFF: no row).
-struct RgHostGroup {
-    uint32_t row[4];   // absolute rows (~0u: none)
-    uint32_t uoff, nu; // union entries [uoff, uoff + nu)
-    uint32_t lo, hi;   // lowest / highest union column
+// Row-group layout of a matrix, built at create for dose_spmv, the batched
+// SpMM, the adjoint and the fused objective pass.  Rows without entries are not
+// stored.  The others are put in an order in which neighbours see the same
+// spots (rg_layout.cu) and cut into groups of up to hr (8, or 4) rows.  A group
+// stores the union of its rows' columns once and, for each union column, the
+// hr rows' stored values side by side (the stored zero where a row has no
+// entry).  A warp takes a whole group: per union column one gather of x feeds
+// hr rows' dot products, and after the residuals are known one
+// read-modify-write of the gradient accumulator adds all rows' contributions.
+//
+// The groups are cut into contiguous runs of about equal cost, one per CTA.  A
+// CTA keeps only the columns its groups see: `dict` lists them (ascending), the
+// stored column indices are positions in that list, and x, the batched X and
+// the gradient accumulators hold one element per listed column.
+//
+// Every warp streams its own packets (runs of whole groups, a few KB each)
+// through its own ring of shared-memory slots with bulk copies, so no warp
+// waits for another.  A packet, 16-byte aligned (rg_packet gives the offsets):
+//   u32 ng, u32 nu (union columns of all its groups), 8 bytes unused
+//   u32 per group: its union columns
+//   u32 x hr per group: its rows (0xFFFFFFFF: none)
+//   f32 x hr per group: their scales (FP8 only)
+//   nu column indices of iw bytes, groups one after the other
+//   nu x hr stored values
+// A group whose union exceeds a packet is cut into pieces of one packet each,
+// whose partial sums are carried from piece to piece (RG_CARRY_*); the earlier
+// pieces come a second time (RG_AGAIN) for the gradient updates.
+enum : uint32_t {
+    RG_SIZE_MASK = 0x00FFFFFFu,  // packet size in 16-byte units
+    RG_FORWARD = 0x01000000u,    // forward passes use this packet
+    RG_SCATTER = 0x02000000u,    // gradient updates use it
+    RG_CARRY_IN = 0x04000000u,   // row sums continue the previous packet's
+    RG_CARRY_OUT = 0x08000000u,  // ... and go on in the next one
+    RG_AGAIN = 0x10000000u,      // an earlier piece, for its gradient updates
+};
+struct RgPacket {
+    uint32_t rows, scales, cols, vals, bytes;
+};
+RgPacket rg_packet(uint32_t ng, uint32_t nu, uint32_t hr, uint32_t iw, uint32_t es, bool scales);
+
+// A call's deal of the packets to warps: warp w of CTA c streams the packets
+// pk[begin[c nw + w] .. begin[c nw + w + 1)), each as its offset / 16, its size /
+// 16 | flags, its first row in row_list and its rows.
+enum { RG_DEAL_SPMV, RG_DEAL_SPMM, RG_DEAL_SPMM_FEW, RG_DEAL_F64, RG_DEAL_FUSED, RG_DEAL_ADJOINT, RG_DEALS };
+struct RgDeal {
+    uint4* pk = nullptr;
+    uint32_t* begin = nullptr;
+    uint32_t nw = 0;
 };
 
 struct RowGroups {
     bool built = false;
-    uint32_t iw = 4;                // bytes per union column index (2 when ncols <= 65536)
-    uint64_t n_union = 0;           // union entries of all groups
-    void* ucol = nullptr;           // union column indices
-    void* uval = nullptr;           // four stored values per union entry
-    uint4* grp = nullptr;           // group records (depend on the stage cut)
+    uint32_t grid = 0;              // CTAs the groups are cut for
+    uint32_t hr = 8;                // rows per group (values stored per union column)
+    uint32_t iw = 4;                // bytes per stored column index (2 when ncols <= 65536)
+    uint32_t order = 0;             // row order taken (rg_layout.cu)
+    bool keep = false;              // the stored-row order of the fused pass (rg_layout.cu), cut for
+    uint32_t keep_nw = 0;           //   this many warps per CTA
+    std::vector<uint32_t> keep_tag; //   each packet's warp
+    uint64_t n_groups = 0, n_union = 0;
+    unsigned char* data = nullptr;  // packets
+    uint32_t* row_list = nullptr;   // the packets' rows once more, packet by packet
+    uint32_t* dict = nullptr;       // columns of each CTA, ascending
+    uint32_t* dict_begin = nullptr; // grid + 1
+    uint32_t* col_ptr = nullptr;    // 8 ncols + 1: where column j lies in dict (and so in g_part): in CTAs
+    uint32_t* col_pos = nullptr;    //   k, k + 8, ... at col_pos[col_ptr[8 j + k] .. col_ptr[8 j + k + 1])
+    uint2* zero_runs = nullptr;     // rows without entries: first row, rows (at most kRgZeroRun)
+    uint32_t n_zero_runs = 0;
     uint32_t* mask = nullptr;       // one bit per row: the row has entries
-    double* f_rows = nullptr;       // objective sums of the finalize's row blocks
-    uint32_t* ticket = nullptr;     // finalize: row blocks done (reset by the last one)
-    uint32_t nblk_rows = 0;         // finalize row blocks (256 rows per warp, 8 warps)
-    DevSchedule sched;              // stages of groups, dealt to CTAs with column windows
-    uint32_t tile_u = 0, tile_g = 0, tile_rows = 0;  // stage limits of the schedule in effect
+    float* g_part = nullptr;        // partial gradients, one element per dict entry
+    RgDeal deal[RG_DEALS];
+    uint32_t wmax = 0;              // most columns of any CTA
+    uint32_t slot = 0;              // bytes of a ring slot (the largest packet)
+    uint32_t tile_u = 0;            // union columns per packet asked for
+    uint64_t data_bytes = 0;        // of the packets
     uint64_t bytes = 0;             // device bytes of the arrays above
-    std::vector<RgHostGroup> host; // kept for re-cutting the stages
+    std::vector<uint4> host_pk;     // the packets in memory order, as in RgDeal
+    std::vector<uint32_t> cta_pk;   // grid + 1: packets of each CTA
+    std::vector<uint32_t> pk_cost;  // dealing cost of each packet
+    std::vector<uint8_t> pk_chain;  // the packet stays with the one before it
 };
 
 // Shape of the adjoint / fused kernels (warp specialisation and pipeline).
@@ -164,11 +210,11 @@ struct AdjTuning {
     // layout of the adjoint / fused passes: 0 = row groups where they apply, else
     // CSR; 1 = CSR; 2 = row groups (create fails if they do not apply)
     uint32_t layout = 0;
-    uint32_t rg_tile_u = 0;        // row groups: union entries per stage (0 = by format)
-    uint32_t rg_tile_rows = 512;   // row groups: rows a stage may span
-    uint32_t rg_stages = 2;        // row groups: pipeline depth
-    uint32_t rg_warps = 0;         // row groups: worker warps (0 = as many as fit, up to kRgMaxWarps)
-    uint32_t rg_l2_prefetch = 0;   // row groups: stages prefetched into L2 ahead of the ring (0 = off)
+    uint32_t rg_tile_u = 0;        // row groups: union columns per packet, at create (0 = kRgDefaultUnion)
+    uint32_t rg_tile_rows = 512;   // row groups: accepted and reported; packets hold at most kRgMaxRows rows
+    uint32_t rg_stages = 2;        // row groups: slots of a gradient warp's ring
+    uint32_t rg_warps = 0;         // row groups: gradient warps (0 = as many as fit, up to kRgMaxWarps)
+    uint32_t rg_l2_prefetch = 0;   // row groups: accepted and reported; the rings need no L2 prefetch
 };
 
 }  // namespace dose
@@ -203,7 +249,8 @@ struct dose_matrix {
 
     dose::SellArrays sell;  // DOSE_CREATE_SELL only
 
-    dose::RowGroups rg;     // row-group layout of the adjoint / fused passes (when it applies)
+    dose::RowGroups rg;     // row-group layout (when it applies)
+    dose::RowGroups rgf;    // ... in the stored-row order, for the fused pass (small matrices, multi-beam plans)
 
     // adjoint scratch: per-CTA partial gradients and objective values
     float* g_part = nullptr;     // adj.grid * ncols
@@ -255,31 +302,33 @@ cudaError_t launch_adjoint(const dose_matrix* A, int mode, const float* x, const
 // Whether the adjoint / fused kernels can run on A (window and accumulators fit;
 // per-row vectors 16-byte aligned); sets the error message if not.
 dose_status adjoint_supported(const dose_matrix* A, bool quad, const float* const* vecs, int nvec);
-// Row-group layout (rg_layout.cu, rg_kernel.cu).  build_row_groups forms the
-// groups from the host CSR and the stored values; false (with *why) if some row
-// does not fit one stage.  rg_schedule cuts the stages and deals them
-// (re-run when the tuning changes).
-bool build_row_groups(dose_matrix* A, const uint32_t* rp, const uint32_t* col, const unsigned char* vals,
-                      std::string* why, cudaError_t* err);
-cudaError_t rg_schedule(dose_matrix* A, const AdjTuning& t);
-void free_row_groups(dose_matrix* A);
-// Worker warps that fit for tuning t (0: none); *smem the dynamic shared memory.
-uint32_t rg_shape(const dose_matrix* A, const AdjTuning& t, bool quad, size_t* smem);
+// Row-group layout (rg_layout.cu).  build_row_groups forms the layout from the
+// host CSR and the stored values; false (with *why) if some row is too long
+// (*err = cudaErrorInvalidValue: longer than the caller's rg_tile_union), or with
+// *err set if memory ran out.  rg_schedule deals the packets to the warps of
+// each call (re-run when the tuning changes).
+bool build_row_groups(dose_matrix* A, RowGroups& R, bool keep, const uint32_t* rp, const uint32_t* col,
+                      const unsigned char* vals, const float* scales, std::string* why, cudaError_t* err);
+cudaError_t rg_schedule(dose_matrix* A);
+void free_row_groups(RowGroups& R);
+const RowGroups& rg_of(const dose_matrix* A, int which);  // the layout call RG_DEAL_* runs on
+// Worker warps of a call (RG_DEAL_*) that fit beside their slots, the depth of
+// their rings and the dynamic shared memory; 0: the call does not fit.
+uint32_t rg_warps(const dose_matrix* A, int which, uint32_t* depth, size_t* smem);
+uint32_t rg_forward_warps(const dose_matrix* A, int which, uint32_t* depth, size_t* smem);  // rg_spmm.cu
+uint32_t rg_gradient_warps(const dose_matrix* A, const AdjTuning& t, bool quad, uint32_t* depth, size_t* smem);  // rg_kernel.cu
 // Whether the adjoint (quad = false) / fused pass of A runs on the row-group layout.
 bool rg_active(const dose_matrix* A, bool quad);
 cudaError_t launch_rg(const dose_matrix* A, int mode, const float* x, const float* p, const float* w,
                       const float* r, float* d, double* f, float* g, float* x_update, float eta, cudaStream_t s);
 uint64_t rg_fused_bytes(const dose_matrix* A, bool with_d);
 // Batched SpMM on the row-group layout (rg_spmm.cu): whether it applies to the
-// matrices A[0 .. count) (count <= kRgSpmmMaxPerLaunch), and the launches.
+// matrices A[0 .. count), and in how many launches.
 constexpr uint32_t kRgSpmmMaxPerLaunch = 32;
-bool rg_spmm_applies(const dose_matrix* const* A, int count, size_t* smem, uint32_t* depth);
-// d = A x on the row-group layout (rg_spmm.cu): whether it fits, and the launch.
-bool rg_spmv_applies(const dose_matrix* A, size_t* smem, uint32_t* depth);
-// dose_spmv_f64 on the row-group layout (rg_spmm.cu): x64 is the handle's
-// prepared x (ncols + 1 elements of 8 bytes, the last one zero).
-bool rg_spmv64_applies(const dose_matrix* A, size_t* smem, uint32_t* depth);
-cudaError_t launch_rg_spmv64(const dose_matrix* A, const void* x64, double* d, bool native, cudaStream_t s);
+bool rg_spmm_applies(const dose_matrix* const* A, int count, int* launches);
+// dose_spmv_f64 on the row-group layout (rg_spmm.cu).
+bool rg_spmv64_applies(const dose_matrix* A);
+cudaError_t launch_rg_spmv64(const dose_matrix* A, const double* x, double* d, bool native, cudaStream_t s);
 // Whether dose_spmv takes the row-group form for this handle (dose_api.cu).
 bool spmv_on_row_groups(const dose_matrix* A);
 cudaError_t launch_rg_spmv(const dose_matrix* A, const float* x, float* d, cudaStream_t s);
@@ -318,10 +367,14 @@ constexpr uint32_t kMaxSmemPerBlock = 227 * 1024;
 __host__ __device__ constexpr uint32_t value_bytes(int fmt) {
     return fmt == DOSE_FMT_FP8E4M3_ROWSCALE ? 1u : (fmt == DOSE_FMT_F32 ? 4u : 2u);
 }
-// Worker warps of the row-group kernel (plus one producer): 16 warps in all, so
-// that each of the SM's four register files holds four warps of up to 128 registers.
+// Row-group layout: worker warps of the gradient kernels (one producer-less CTA per SM).
 constexpr uint32_t kRgMaxWarps = 15;
-constexpr uint32_t kRgMaxUnionReg = 320;  // union columns a group may hold to stay in registers
+constexpr uint32_t kRgDefaultUnion = 320;  // union columns of a packet (6 KB with eight 16-bit values each)
+constexpr uint32_t kRgMaxRows = 64;        // rows of a packet
+constexpr uint32_t kRgZeroRun = 1024;      // rows of a run without entries
+// The fused pass keeps the stored-row order up to this many rows with entries (rg_layout.cu):
+// beyond, another order moves f by at most 4e-10 of itself (measured on beams of 0.5 to 7e5 rows)
+constexpr uint32_t kRgKeepRows = 200000;
 constexpr uint32_t kMaxAdjWarps = 20;      // producer + forward + scatter warps of the adjoint kernels
 constexpr uint32_t kSellDefaultSigma = 1u << 20;  // rows per sorting window of the SELL copy
 constexpr uint32_t kAdjMinScatterWarps = 8;

@@ -53,14 +53,7 @@ template <int MODE>
 __global__ void prepare_x_kernel(const double* __restrict__ x, uint2* __restrict__ out, uint32_t n) {
     const uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j > n) return;
-    const double v = j < n ? x[j] : 0.0;
-    if (MODE == F64_DF) {
-        const float hi = __double2float_rn(v);
-        const float lo = __double2float_rn(v - (double)hi);  // v - hi is exact in FP64
-        out[j] = make_uint2(__float_as_uint(hi), __float_as_uint(lo));
-    } else {
-        out[j] = make_uint2((uint32_t)__double2loint(v), (uint32_t)__double2hiint(v));
-    }
+    out[j] = prepare_x<MODE>(j < n ? x[j] : 0.0);
 }
 
 // Lane li of an L-lane group takes the groups of four consecutive entries at
@@ -289,8 +282,17 @@ bool spmv_f64_x_in_smem(const dose_matrix* A) {
     return spmv_x_cols(A) > 0 && spmv_f64_smem_bytes(A, true) <= kMaxSmemPerBlock;
 }
 
+// The row-group form: where dose_spmv takes it too.  FP64 FMAs only when the
+// caller asks for it (fwd_layout = 2): they are bound by the FP64 pipe, and the
+// layout stores more values than the matrix has entries.
+static bool spmv_f64_on_row_groups(const dose_matrix* A, bool native) {
+    return (A->fwd.tuning.layout == 2 || !native) && !(A->flags & DOSE_CREATE_SELL) && spmv_on_row_groups(A) &&
+           rg_spmv64_applies(A);
+}
+
 cudaError_t launch_spmv_f64(const dose_matrix* A, const double* x, double* d, bool native, cudaStream_t s) {
     if (A->nrows == 0) return cudaSuccess;
+    if (spmv_f64_on_row_groups(A, native)) return launch_rg_spmv64(A, x, d, native, s);
     const uint32_t nx = A->ncols + 1;
     if (native)
         prepare_x_kernel<F64_DP><<<(nx + 255) / 256, 256, 0, s>>>(x, A->x64, A->ncols);
@@ -298,12 +300,6 @@ cudaError_t launch_spmv_f64(const dose_matrix* A, const double* x, double* d, bo
         prepare_x_kernel<F64_DF><<<(nx + 255) / 256, 256, 0, s>>>(x, A->x64, A->ncols);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    // the row-group form only when the caller asks for it (fwd_layout = 2): this
-    // kernel is bound by its arithmetic, not its bytes, and the layout's 1.17
-    // stored values per entry cost more than its fewer bytes save (clinical
-    // beam, F16: 0.228 ms on row groups against 0.221 ms on CSR)
-    if (A->fwd.tuning.layout == 2 && spmv_on_row_groups(A) && rg_spmv64_applies(A, nullptr, nullptr))
-        return launch_rg_spmv64(A, A->x64, d, native, s);
     Spmv64Params p;
     const bool idx16 = (A->flags & DOSE_CREATE_U16_INDEX) != 0;
     p.row_ptr = A->row_ptr;
