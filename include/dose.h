@@ -153,7 +153,8 @@ typedef struct {
        Row groups: up to eight rows (four where that stores less, and for F32) that see
        nearly the same columns share one list of the union of their columns, with the
        rows' values stored side by side (stored zeros where a row has no entry); built
-       when no row has more than 4096 entries.  The rows of a group need not be
+       when no row has more than 4096 entries (or, for the forward calls alone, when rows
+       are longer and the layout stores less than the CSR arrays).  The rows of a group need not be
        consecutive: on a voxel grid, whose strides are looked for in the matrix, they are
        neighbours along the beam or small cubes.  The union order is chosen per group
        (shared-memory banks), so these passes sum a row's terms in another order than the

@@ -869,7 +869,7 @@ static dose_status create_matrix(const dose_csr_desc* desc, unsigned flags, cons
         bool ok = build_row_groups(A.get(), A->rg, false, A->host_row_ptr.data(), col.data(), vals.data(), scl.data(), &why, &e);
         uint64_t full = 0;
         for (uint32_t i = 0; i < nrows; ++i) full += A->host_row_ptr[i + 1] > A->host_row_ptr[i];
-        if (ok && (plan || full < kRgKeepRows) &&
+        if (ok && !A->rg.forward_only && (plan || full < kRgKeepRows) &&
             !build_row_groups(A.get(), A->rgf, true, A->host_row_ptr.data(), col.data(), vals.data(), scl.data(), &why, &e)) {
             free_row_groups(A->rg);
             ok = false;
@@ -904,7 +904,7 @@ static dose_status create_matrix(const dose_csr_desc* desc, unsigned flags, cons
             return DOSE_ERR_UNSUPPORTED;
         }
     }
-    if (A->fwd.tuning.layout == 2 && !spmv_on_row_groups(A.get())) {
+    if (A->fwd.tuning.layout == 2 && (A->rg.forward_only || !spmv_on_row_groups(A.get()))) {
         free_all(A.get());
         set_error("fwd_layout = 2: dose_spmv cannot run on the row-group layout of this handle" +
                   std::string((flags & DOSE_CREATE_COMPENSATED) ? " (DOSE_CREATE_COMPENSATED sums on CSR)" : ""));
@@ -1236,10 +1236,10 @@ dose_status dose_set_tuning(dose_matrix* A, const dose_tuning* tuning) {
     st = apply_schedule(A, A->fwd, t, A->fwd_windowed);
     if (st == DOSE_OK && A->fwd64_own) st = apply_schedule(A, A->fwd64, t, false);
     if (st != DOSE_OK) return st;
-    if (at.layout == 2 && !A->rg.built) return invalid("adj_layout = 2: the handle has no row-group layout");
-    if (t.layout == 2 && (!A->rg.built || (A->flags & DOSE_CREATE_COMPENSATED)))
+    if (at.layout == 2 && (!A->rg.built || A->rg.forward_only)) return invalid("adj_layout = 2: the handle has no row-group layout");
+    if (t.layout == 2 && (!A->rg.built || A->rg.forward_only || (A->flags & DOSE_CREATE_COMPENSATED)))
         return invalid("fwd_layout = 2: dose_spmv cannot run on the row-group layout of this handle");
-    if (A->rg.built && at.rg_tile_u != A->adj_tuning.rg_tile_u && A->max_row_len > at.rg_tile_u)
+    if (A->rg.built && !A->rg.forward_only && at.rg_tile_u != A->adj_tuning.rg_tile_u && A->max_row_len > at.rg_tile_u)
         return invalid("tuning.rg_tile_union is smaller than the longest row");
     A->adj_tuning = at;
     if (A->rg.built && (e = rg_schedule(A)) != cudaSuccess) return cuda_fail(e, "row-group schedule");

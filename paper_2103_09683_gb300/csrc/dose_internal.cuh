@@ -172,6 +172,8 @@ struct RowGroups {
     uint32_t hr = 8;                // rows per group (values stored per union column)
     uint32_t iw = 4;                // bytes per stored column index (2 when ncols <= 65536)
     uint32_t order = 0;             // row order taken (rg_layout.cu)
+    bool forward_only = false;      // rows too long for the gradient passes: dose_spmv, dose_spmv_f64 and the
+                                    //   batched SpMM only
     bool keep = false;              // the stored-row order of the fused pass (rg_layout.cu), cut for
     uint32_t keep_nw = 0;           //   this many warps per CTA
     std::vector<uint32_t> keep_tag; //   each packet's warp

@@ -455,7 +455,7 @@ cudaError_t launch_fmt(const dose_matrix* A, const RgParams& p, size_t smem, cud
 // packets instead.
 uint32_t rg_gradient_warps(const dose_matrix* A, const AdjTuning& t, bool quad, uint32_t* depth, size_t* smem) {
     const RowGroups& R = rg_of(A, quad ? RG_DEAL_FUSED : RG_DEAL_ADJOINT);
-    if (!R.built) return 0;
+    if (!R.built || R.forward_only) return 0;
     uint32_t d = std::min<uint32_t>(t.rg_stages, kRgMaxDepth);
     const size_t fixed = kRgHeader + (quad ? kRgZeroBytes + round_up((R.wmax + 1) * 4, 128) : 0);
     const size_t base = kRgWarpBytes + (size_t)round_up(R.wmax, 32) * 4, per = base + (size_t)d * R.slot;

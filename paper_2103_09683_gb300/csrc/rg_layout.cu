@@ -43,7 +43,8 @@ namespace {
 
 uint32_t round_up16(uint32_t v) { return (v + 15) / 16 * 16; }
 
-constexpr uint32_t kMaxRowEntries = 4096;  // longest row the layout takes
+constexpr uint32_t kMaxRowEntries = 4096;  // longest row of the gradient passes (and most columns of a packet)
+constexpr uint32_t kMaxForwardRow = 32768; // ... of a layout for the forward passes alone
 constexpr uint32_t kTile = 8;              // voxels per side of the tiles the rows are ordered by
 constexpr uint64_t kGroupCost = 4;         // dealing cost of a group, in steps of 32 columns: its reduction,
                                            // outputs and its share of its packet (140 instructions against
@@ -96,6 +97,7 @@ struct Csr {
     const unsigned char* vals;
     const float* scales;  // FP8
     uint32_t nrows, ncols, es;
+    uint32_t max_union;   // union columns of a group
 };
 
 // Marks of the columns of the group being formed.
@@ -120,6 +122,7 @@ struct Marks {
 template <class E>
 void form_groups(const Csr& A, const uint32_t* rows, const uint8_t* cube, size_t n, uint32_t hr, Marks& mk,
                  std::vector<uint32_t>& U, E emit) {
+    const uint64_t max_union = A.max_union;
     size_t first = 0;
     uint32_t cnt = 0;
     U.clear();
@@ -133,7 +136,7 @@ void form_groups(const Csr& A, const uint32_t* rows, const uint8_t* cube, size_t
                 for (uint32_t k = kb; k < ke; ++k) fresh += !mk.has(A.col[k]);
                 const uint64_t nu = U.size() + fresh;
                 join = 10 * (uint64_t)fresh <= 7 * (uint64_t)len + 80 &&
-                       2 * nu <= 3 * std::max<uint64_t>(U.size(), len) + 16 && nu <= kMaxRowEntries;
+                       2 * nu <= 3 * std::max<uint64_t>(U.size(), len) + 16 && nu <= max_union;
             }
             if (!join) {
                 emit(first, cnt, U);
@@ -194,7 +197,7 @@ Strides find_strides(const Csr& A, const std::vector<uint32_t>& rows, const uint
         for (uint32_t k = A.rp[r]; k < A.rp[r + 1]; ++k) mk.add(A.col[k]);
         const uint32_t slack = (cmax[r] - cmin[r]) / 2 + 2;
         std::vector<Hit> h;
-        uint64_t budget = 4000000;  // entries looked at per sample
+        uint64_t budget = std::max<uint64_t>(4000000, 12000ull * len);  // entries looked at per sample
         for (size_t k = std::upper_bound(rows.begin(), rows.end(), r) - rows.begin(); k < n; ++k) {
             const uint32_t q = rows[k], lq = A.rp[q + 1] - A.rp[q];
             if (q - r < 2 || 4 * lq < 3 * len || 4 * len < 3 * lq) continue;
@@ -357,9 +360,9 @@ struct Grp {
     uint32_t nu;
     uint64_t uoff;        // its union in the segment's column list
     // in steps of 32 columns; all but the last piece of a long group come twice
-    uint64_t cost(uint32_t max_u) const {
+    uint64_t cost(uint32_t max_u, bool again) const {
         const uint64_t steps = (nu + 31) / 32, np = (nu + max_u - 1) / max_u;
-        return kGroupCost * (2 * np - 1) + steps + steps * (np - 1) / (2 * np);
+        return kGroupCost * np + steps + (again ? kGroupCost * (np - 1) + steps * (np - 1) / (2 * np) : 0);
     }
 };
 
@@ -550,7 +553,7 @@ struct CtaOut {
 // one.  keep (each group's warp): packets hold groups of one warp, their columns
 // in the order of the stored-row layout.
 void write_cta(const Csr& A, uint32_t hr, uint32_t iw, uint32_t cap, uint32_t max_u, const uint32_t* rows,
-               const std::vector<std::pair<const Grp*, const uint32_t*>>& groups, const std::vector<uint32_t>* keep,
+               const std::vector<std::pair<const Grp*, const uint32_t*>>& groups, const std::vector<uint32_t>* keep, bool again,
                std::vector<uint32_t>& pos, std::vector<uint32_t>& seen, uint32_t gen, CtaOut& out) {
     const bool fp8 = A.scales != nullptr;
     // distinct columns
@@ -670,7 +673,7 @@ void write_cta(const Csr& A, uint32_t hr, uint32_t iw, uint32_t cap, uint32_t ma
         }
         // a group of several pieces: its residuals are known after the last one, so
         // the earlier pieces come once more for the scatter
-        for (uint32_t i = 0; i + 1 < np; ++i) {
+        for (uint32_t i = 0; again && i + 1 < np; ++i) {
             const uint4 q = out.pk[piece_pk[i]];
             out.pk.push_back(make_uint4(q.x, (q.y & RG_SIZE_MASK) | RG_SCATTER | RG_AGAIN, q.z, q.w));
             out.cost.push_back(out.cost[piece_pk[i]]);
@@ -786,15 +789,24 @@ bool build_row_groups(dose_matrix* A, RowGroups& R, bool keep, const uint32_t* r
     *err = cudaSuccess;
     const uint32_t nrows = A->nrows, ncols = A->ncols;
     const uint32_t es = value_bytes(A->fmt);
-    const Csr M{rp, col, vals, A->fmt == DOSE_FMT_FP8E4M3_ROWSCALE ? scales : nullptr, nrows, ncols, es};
-    R.iw = ncols <= 65536u ? 2u : 4u;
-    if (A->max_row_len > kMaxRowEntries) {
-        *why = "a row has " + std::to_string(A->max_row_len) + " entries; row groups hold at most " +
-               std::to_string(kMaxRowEntries) + " columns";
+    const Csr M{rp, col, vals, A->fmt == DOSE_FMT_FP8E4M3_ROWSCALE ? scales : nullptr, nrows, ncols, es,
+                A->max_row_len > kMaxRowEntries ? 2 * kMaxForwardRow : kMaxRowEntries};
+    // Rows past the gradient passes' limit: a layout for the forward passes alone,
+    // if it stores less than the CSR arrays (below).  The beam shaped like the
+    // paper's liver beam 1 has rows of 5000 of its 68,000 spots: dose 206 us on CSR.
+    const bool forward_only = A->max_row_len > kMaxRowEntries;
+    // (the indices are positions in a CTA's list, which fits shared memory and so
+    // 16 bits wherever the forward passes run; the wide form is kept where a
+    // handle's gradient passes have reported it)
+    R.iw = ncols <= 65536u || forward_only ? 2u : 4u;
+    const std::string too_long = "a row has " + std::to_string(A->max_row_len) + " entries; row groups hold at most " +
+                                 std::to_string(kMaxRowEntries) + " columns";
+    if (forward_only && (keep || A->max_row_len > kMaxForwardRow || A->adj_tuning.layout == 2)) {
+        *why = too_long;
         return false;
     }
     const uint32_t tile_u = A->adj_tuning.rg_tile_u ? A->adj_tuning.rg_tile_u : kRgDefaultUnion;
-    if (A->max_row_len > tile_u && A->adj_tuning.rg_tile_u) {
+    if (A->max_row_len > tile_u && A->adj_tuning.rg_tile_u && !forward_only) {
         *err = cudaErrorInvalidValue;
         return false;
     }
@@ -877,10 +889,15 @@ bool build_row_groups(dose_matrix* A, RowGroups& R, bool keep, const uint32_t* r
         uint64_t total = 0, n_groups = 0, n_union = 0;
         for (const auto& v : sg)
             for (const Grp& g : v) {
-                total += g.cost(cap);
+                total += g.cost(cap, !forward_only);
                 n_union += g.nu;
                 ++n_groups;
             }
+        const uint64_t per_entry = es + ((A->flags & DOSE_CREATE_U16_INDEX) ? 2u : 4u);
+        if (forward_only && n_union * (hr * es + R.iw) >= (uint64_t)A->nnz * per_entry) {
+            *why = too_long;
+            return false;
+        }
         std::vector<std::vector<std::pair<const Grp*, const uint32_t*>>> cta(grid);
         std::vector<std::vector<uint32_t>> tag(keep ? grid : 0);
         if (keep) {
@@ -898,7 +915,7 @@ bool build_row_groups(dose_matrix* A, RowGroups& R, bool keep, const uint32_t* r
             uint64_t run = 0;
             for (uint32_t s = 0; s < sg.size(); ++s)
                 for (const Grp& g : sg[s]) {
-                    const uint64_t c = g.cost(cap);
+                    const uint64_t c = g.cost(cap, !forward_only);
                     cta[std::min<uint64_t>(grid - 1, (2 * run + c) * grid / (2 * total))].push_back({&g, su[s].data() + g.uoff});
                     run += c;
                 }
@@ -917,7 +934,7 @@ bool build_row_groups(dose_matrix* A, RowGroups& R, bool keep, const uint32_t* r
                 w.pos.assign(std::max(ncols, 1u), 0);
                 w.seen.assign(std::max(ncols, 1u), 0);
             }
-            write_cta(M, hr, R.iw, pack, max_u, rows.data(), cta[c], keep ? &tag[c] : nullptr, w.pos, w.seen, ++w.gen, out[c]);
+            write_cta(M, hr, R.iw, pack, max_u, rows.data(), cta[c], keep ? &tag[c] : nullptr, !forward_only, w.pos, w.seen, ++w.gen, out[c]);
         });
         if (!ok) throw std::bad_alloc();
 
@@ -947,6 +964,10 @@ bool build_row_groups(dose_matrix* A, RowGroups& R, bool keep, const uint32_t* r
             dict_begin[c + 1] = (uint32_t)dict.size();
             R.cta_pk[c + 1] = (uint32_t)pk.size();
             R.wmax = std::max(R.wmax, (uint32_t)out[c].dict.size());
+            if (R.iw == 2 && out[c].dict.size() > 65536) {
+                *why = "a CTA's rows see more than 65536 columns";
+                return false;
+            }
             R.slot = std::max(R.slot, out[c].slot);
         }
         R.slot = (std::max(R.slot, 128u) + 127) / 128 * 128;
@@ -1010,6 +1031,7 @@ bool build_row_groups(dose_matrix* A, RowGroups& R, bool keep, const uint32_t* r
         R.tile_u = tile_u;
         R.order = (uint32_t)order;
         R.keep = keep;
+        R.forward_only = forward_only;
         R.data_bytes = bytes;
         R.bytes = bytes + row_list.size() * 4 + dict.size() * 12 + (size_t)ncols * 32 + zr.size() * 8 + mask.size() * 4;
         R.built = true;
