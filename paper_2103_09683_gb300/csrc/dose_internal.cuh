@@ -323,6 +323,11 @@ uint32_t rg_gradient_warps(const dose_matrix* A, const AdjTuning& t, bool quad, 
 bool rg_active(const dose_matrix* A, bool quad);
 cudaError_t launch_rg(const dose_matrix* A, int mode, const float* x, const float* p, const float* w,
                       const float* r, float* d, double* f, float* g, float* x_update, float eta, cudaStream_t s);
+// The fused passes of n scenarios (f[k], g + k ncols) overlapped, with one
+// finalize: whether that applies, and the launches.
+bool rg_chain_applies(const dose_matrix* const* A, uint32_t n);
+cudaError_t launch_rg_chain(const dose_matrix* const* A, uint32_t n, const float* x, const float* p, const float* w,
+                            double* f, float* g, cudaStream_t s);
 uint64_t rg_fused_bytes(const dose_matrix* A, bool with_d);
 // Batched SpMM on the row-group layout (rg_spmm.cu): whether it applies to the
 // matrices A[0 .. count), and in how many launches.

@@ -29,13 +29,13 @@ constexpr uint32_t kRgZeroBytes = 4096;    // zeros that the bulk stores of rows
 // A row-group kernel's launch, as a programmatic dependent of what is before it
 // in the stream (early) or an ordinary one.
 template <class K, class P>
-cudaError_t rg_launch(K k, const P& p, uint32_t grid, uint32_t threads, size_t smem, cudaStream_t s, bool early = true) {
+cudaError_t rg_launch(K k, const P& p, dim3 grid, uint32_t threads, size_t smem, cudaStream_t s, bool early = true) {
     if (smem > 48 * 1024) {
         const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
+    cfg.gridDim = grid;
     cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;

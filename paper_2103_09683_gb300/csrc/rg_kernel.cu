@@ -32,6 +32,7 @@
 namespace dose {
 namespace {
 
+constexpr uint32_t kRgMaxChain = 64;                // passes of one chain
 constexpr uint32_t kRgRowWarps = 3;                 // warps of the rows without entries
 constexpr uint32_t kRgWarpBytes = kRgMaxRows * 4;   // a worker's row buffer: row sums, then residuals
 
@@ -45,8 +46,17 @@ struct RgParams {
     double* f_part;    // grid
     const uint32_t* mask;  // rows with entries
     uint32_t wmax, nw, depth, slot;
+    uint32_t chain;        // RG_CHAIN_*
     int* err;
 };
+
+// Passes of different matrices that only share their inputs (the scenarios of a
+// robust objective) may overlap: each lets the next start once the kernels before
+// the first are done (so the next need not wait for anything), its CTAs take the
+// SMs that the previous pass's have left, and it waits for the previous pass only
+// before it ends, so that the last one's end is the end of all.
+constexpr uint32_t RG_CHAIN_NEXT = 1;   // let the next pass start early
+constexpr uint32_t RG_CHAIN_PREV = 2;   // started early: wait at the end
 
 // Row numbers and per-row vectors of a warp's packets, ahead of their use: the
 // packets with any flag of NEED, in the order the stream delivers them.  Lane l
@@ -252,7 +262,8 @@ __global__ void __launch_bounds__((kRgMaxWarps + kRgRowWarps) * 32, 1) rg_kernel
     const uint32_t db = C.db, nc = C.nc;
     float4* g4 = reinterpret_cast<float4*>(gacc);
     for (uint32_t j = t; j < NW * gstride / 4; j += T) g4[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-    rg_wait_previous();
+    if (!(p.chain & RG_CHAIN_PREV)) rg_wait_previous();
+    if (p.chain & RG_CHAIN_NEXT) rg_let_next_start();
     if (QUAD) {
         C.each(t, T, [&](uint32_t j, uint32_t c) { xs[j] = __ldg(p.x + c); });
         if (t == 0) xs[nc] = 0.f;
@@ -345,7 +356,7 @@ __global__ void __launch_bounds__((kRgMaxWarps + kRgRowWarps) * 32, 1) rg_kernel
         for (uint32_t o = 16; o > 0; o >>= 1) f_lane += __shfl_xor_sync(0xffffffffu, f_lane, o);
         if (lane == 0) fred[warp] = f_lane;
     }
-    rg_let_next_start();
+    if (!(p.chain & RG_CHAIN_NEXT)) rg_let_next_start();
     __syncthreads();
     for (uint32_t j = t; j < nc; j += T) {
         float sum = gacc[j];
@@ -357,6 +368,7 @@ __global__ void __launch_bounds__((kRgMaxWarps + kRgRowWarps) * 32, 1) rg_kernel
         for (uint32_t w2 = 0; w2 < NW + kRgRowWarps; ++w2) sum += fred[w2];
         p.f_part[cta] = sum;
     }
+    if (p.chain & RG_CHAIN_PREV) rg_wait_previous();
 }
 
 // Second kernel of the row-group passes: column block cb: g_j = s * (sum of the partials of the CTAs that see column j, in CTA
@@ -375,7 +387,14 @@ struct RgFin {
     double* f;
 };
 
-__global__ void __launch_bounds__(256) rg_finalize(const RgFin q) {
+template <uint32_t N>
+struct RgFins {
+    RgFin q[N];  // block row y finishes pass y
+};
+
+template <uint32_t N>
+__global__ void __launch_bounds__(256) rg_finalize(const __grid_constant__ RgFins<N> all) {
+    const RgFin& q = all.q[blockIdx.y];
     __shared__ float part[8][33];
     __shared__ double red[256];
     const uint32_t w = threadIdx.x >> 5, lane = threadIdx.x & 31, j = blockIdx.x * 32 + lane;
@@ -490,30 +509,32 @@ uint64_t rg_adjoint_bytes(const dose_matrix* A) {
     return A->rg.data_bytes + 4ull * A->nrows + 4ull * A->ncols + rg_parts(A->rg);
 }
 
-cudaError_t launch_rg(const dose_matrix* A, int mode, const float* x, const float* p, const float* w, const float* r,
-                      float* d, double* f, float* g, float* x_update, float eta, cudaStream_t s) {
-    const bool quad = mode == ADJ_MODE_QUADRATIC;
+static cudaError_t launch_main(const dose_matrix* A, bool quad, const float* x, const float* p, const float* w,
+                               const float* r, float* d, uint32_t chain, cudaStream_t s) {
     const int which = quad ? RG_DEAL_FUSED : RG_DEAL_ADJOINT;
     const RowGroups& R = rg_of(A, which);
     size_t smem = 0;
     RgParams prm;
     prm.nw = rg_gradient_warps(A, A->adj_tuning, quad, &prm.depth, &smem);
     if (!prm.nw || R.deal[which].nw != prm.nw) return cudaErrorInvalidConfiguration;
-    if (A->nrows > 0) {
-        prm.A = rg_view(A, which);
-        prm.x = x;
-        prm.v0 = quad ? p : r;
-        prm.v1 = w;
-        prm.d = d;
-        prm.g_part = R.g_part;
-        prm.f_part = A->f_part;
-        prm.mask = R.mask;
-        prm.wmax = R.wmax;
-        prm.slot = R.slot;
-        prm.err = A->err;
-        const cudaError_t e = quad ? launch_fmt<ADJ_MODE_QUADRATIC>(A, prm, smem, s) : launch_fmt<ADJ_MODE_ADJOINT>(A, prm, smem, s);
-        if (e != cudaSuccess) return e;
-    }
+    if (A->nrows == 0) return cudaSuccess;
+    prm.A = rg_view(A, which);
+    prm.x = x;
+    prm.v0 = quad ? p : r;
+    prm.v1 = w;
+    prm.d = d;
+    prm.g_part = R.g_part;
+    prm.f_part = A->f_part;
+    prm.mask = R.mask;
+    prm.wmax = R.wmax;
+    prm.slot = R.slot;
+    prm.chain = chain;
+    prm.err = A->err;
+    return quad ? launch_fmt<ADJ_MODE_QUADRATIC>(A, prm, smem, s) : launch_fmt<ADJ_MODE_ADJOINT>(A, prm, smem, s);
+}
+
+static RgFin finish_of(const dose_matrix* A, bool quad, double* f, float* g, float* x_update, float eta) {
+    const RowGroups& R = rg_of(A, quad ? RG_DEAL_FUSED : RG_DEAL_ADJOINT);
     RgFin q;
     q.g_part = R.g_part;
     q.col_ptr = R.col_ptr;
@@ -526,10 +547,50 @@ cudaError_t launch_rg(const dose_matrix* A, int mode, const float* x, const floa
     q.eta = eta;
     q.f_part = A->f_part;
     q.f = quad ? f : nullptr;
+    return q;
+}
+
+template <uint32_t N>
+static cudaError_t launch_finish(const RgFins<N>& q, uint32_t n, bool early, cudaStream_t s) {
+    const uint32_t nc = q.q[0].ncols;
+    return rg_launch(rg_finalize<N>, q, dim3(nc ? (nc + 31) / 32 : 1, n), 256, 0, s, early);
+}
+
+cudaError_t launch_rg(const dose_matrix* A, int mode, const float* x, const float* p, const float* w, const float* r,
+                      float* d, double* f, float* g, float* x_update, float eta, cudaStream_t s) {
+    const bool quad = mode == ADJ_MODE_QUADRATIC;
+    const cudaError_t e = launch_main(A, quad, x, p, w, r, d, 0, s);
+    if (e != cudaSuccess) return e;
+    RgFins<1> q;
+    q.q[0] = finish_of(A, quad, f, g, x_update, eta);
     // early after the adjoint (18.7 -> 16.8 us on a plan of 780 spots); after the
     // fused pass, whose CTAs leave no registers for a block of this kernel, an
     // ordinary launch: waiting there early cost 14 us (27 -> 41 us, same plan)
-    return rg_launch(rg_finalize, q, A->ncols ? (A->ncols + 31) / 32 : 1, 256, 0, s, !quad);
+    return launch_finish(q, 1, !quad, s);
+}
+
+// The fused passes of n matrices of one shape, overlapped where they may be
+// (distinct matrices, all on this layout, none empty); false: not applicable.
+bool rg_chain_applies(const dose_matrix* const* A, uint32_t n) {
+    if (n < 2 || n > kRgMaxChain) return false;
+    for (uint32_t k = 0; k < n; ++k) {
+        if (!rg_active(A[k], true) || !A[k]->nrows) return false;
+        for (uint32_t j = 0; j < k; ++j)
+            if (A[j] == A[k]) return false;  // they would share one set of partials
+    }
+    return true;
+}
+
+cudaError_t launch_rg_chain(const dose_matrix* const* A, uint32_t n, const float* x, const float* p, const float* w,
+                            double* f, float* g, cudaStream_t s) {
+    RgFins<kRgMaxChain> q;
+    for (uint32_t k = 0; k < n; ++k) {
+        const cudaError_t e = launch_main(A[k], true, x, p, w, nullptr, nullptr,
+                                          (k + 1 < n ? RG_CHAIN_NEXT : 0) | (k ? RG_CHAIN_PREV : 0), s);
+        if (e != cudaSuccess) return e;
+        q.q[k] = finish_of(A[k], true, f + k, g + (size_t)k * A[k]->ncols, nullptr, 0.f);
+    }
+    return launch_finish(q, n, false, s);
 }
 
 }  // namespace dose

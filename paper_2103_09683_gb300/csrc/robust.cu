@@ -96,7 +96,12 @@ dose_status robust_run(const dose_scenarios* S, int mode, const float* x, const 
     }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const uint32_t n = (uint32_t)S->A.size();
-    for (uint32_t k = 0; k < n; ++k) {
+    const bool chain = rg_chain_applies(S->A.data(), n);
+    if (chain) {
+        const cudaError_t e = launch_rg_chain(S->A.data(), n, x, p, w, S->f_s, S->g_s, s);
+        if (e != cudaSuccess) return cuda_fail(e, "robust: scenario passes");
+    }
+    for (uint32_t k = 0; k < n && !chain; ++k) {
         cudaError_t e = launch_adjoint(S->A[k], ADJ_MODE_QUADRATIC, x, p, w, nullptr, nullptr, S->f_s + k,
                                        S->g_s + (size_t)k * S->ncols, nullptr, 0.f, s);
         if (e != cudaSuccess) return cuda_fail(e, "robust: scenario pass");
