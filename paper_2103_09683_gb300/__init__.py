@@ -223,24 +223,48 @@ def _torch():
     return torch
 
 
-def _stream_handle(stream):
-    torch = _torch()
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+# A compute call's host path: on a small matrix the kernel takes about 6 us and
+# the call through this binding took 19 us of host time on a Grace core, most of
+# it in building a Stream object, ctypes pointer objects, imports and the
+# loader's lock.  The helpers below pass plain integers instead.
+
+def _fast():
+    """The loaded library (no lock once it is loaded)."""
+    return _lib if _lib is not None else load()
 
 
-def _dptr(t, dtype, n=None, what="tensor"):
-    """Device pointer of a contiguous CUDA tensor of the given dtype (and length)."""
-    torch = _torch()
-    if not isinstance(t, torch.Tensor) or not t.is_cuda:
+def _raw_stream(stream):
+    """cudaStream_t of a stream (None: the current device's current stream) as an int."""
+    if stream is not None:
+        return stream.cuda_stream
+    c = _torch()._C
+    try:
+        return c._cuda_getCurrentRawStream(c._cuda_getDevice())
+    except AttributeError:  # a torch without these accessors
+        return _torch().cuda.current_stream().cuda_stream
+
+
+def _ptr(t, dtype, n=None, what="tensor"):
+    """Device address of a contiguous CUDA tensor of the given dtype (and length), 0 if empty."""
+    if not isinstance(t, _torch().Tensor) or not t.is_cuda:
         raise TypeError(f"{what} must be a CUDA tensor")
     if t.dtype != dtype:
         raise TypeError(f"{what} must be {dtype}, got {t.dtype}")
     if not t.is_contiguous():
         raise ValueError(f"{what} must be contiguous")
-    if n is not None and t.numel() != n:
-        raise ValueError(f"{what} has {t.numel()} elements, expected {n}")
-    return ctypes.c_void_p(t.data_ptr()) if t.numel() else ctypes.c_void_p(0)
+    have = t.numel()
+    if n is not None and have != n:
+        raise ValueError(f"{what} has {have} elements, expected {n}")
+    return t.data_ptr() if have else 0
+
+
+def _stream_handle(stream):
+    return ctypes.c_void_p(_raw_stream(stream))
+
+
+def _dptr(t, dtype, n=None, what="tensor"):
+    """As _ptr, as a ctypes pointer."""
+    return ctypes.c_void_p(_ptr(t, dtype, n, what))
 
 
 def selftest_bounded_wait(limit_us: int = 20000, stream=None) -> int:
@@ -403,8 +427,10 @@ class DoseMatrix:
         torch = _torch()
         if d is None:
             d = torch.empty(self.nrows, dtype=torch.float32, device=x.device)
-        _check(load().dose_spmv(self._h, _dptr(x, torch.float32, self.ncols, "x"),
-                                _dptr(d, torch.float32, self.nrows, "d"), _stream_handle(stream)))
+        st = _fast().dose_spmv(self._h, _ptr(x, torch.float32, self.ncols, "x"),
+                               _ptr(d, torch.float32, self.nrows, "d"), _raw_stream(stream))
+        if st:
+            _check(st)
         return d
 
     def spmv_f64(self, x, d=None, native: bool = False, stream=None):
@@ -414,9 +440,11 @@ class DoseMatrix:
         torch = _torch()
         if d is None:
             d = torch.empty(self.nrows, dtype=torch.float64, device=x.device)
-        _check(load().dose_spmv_f64(self._h, _dptr(x, torch.float64, self.ncols, "x"),
-                                    _dptr(d, torch.float64, self.nrows, "d"),
-                                    SPMV_F64_NATIVE if native else 0, _stream_handle(stream)))
+        st = _fast().dose_spmv_f64(self._h, _ptr(x, torch.float64, self.ncols, "x"),
+                                   _ptr(d, torch.float64, self.nrows, "d"),
+                                   SPMV_F64_NATIVE if native else 0, _raw_stream(stream))
+        if st:
+            _check(st)
         return d
 
     def adjoint(self, r, g=None, stream=None):
@@ -424,8 +452,10 @@ class DoseMatrix:
         torch = _torch()
         if g is None:
             g = torch.empty(self.ncols, dtype=torch.float32, device=r.device)
-        _check(load().dose_adjoint(self._h, _dptr(r, torch.float32, self.nrows, "r"),
-                                   _dptr(g, torch.float32, self.ncols, "g"), _stream_handle(stream)))
+        st = _fast().dose_adjoint(self._h, _ptr(r, torch.float32, self.nrows, "r"),
+                                  _ptr(g, torch.float32, self.ncols, "g"), _raw_stream(stream))
+        if st:
+            _check(st)
         return g
 
     def fwd_adj_quadratic(self, x, p, w, d=None, f=None, g=None, stream=None, want_d=False):
@@ -438,11 +468,13 @@ class DoseMatrix:
             g = torch.empty(self.ncols, dtype=torch.float32, device=dev)
         if d is None and want_d:
             d = torch.empty(self.nrows, dtype=torch.float32, device=dev)
-        dptr = _dptr(d, torch.float32, self.nrows, "d") if d is not None else None
-        _check(load().dose_fwd_adj_quadratic(
-            self._h, _dptr(x, torch.float32, self.ncols, "x"), _dptr(p, torch.float32, self.nrows, "p"),
-            _dptr(w, torch.float32, self.nrows, "w"), dptr, _dptr(f, torch.float64, 1, "f"),
-            _dptr(g, torch.float32, self.ncols, "g"), _stream_handle(stream)))
+        dptr = _ptr(d, torch.float32, self.nrows, "d") if d is not None else None
+        st = _fast().dose_fwd_adj_quadratic(
+            self._h, _ptr(x, torch.float32, self.ncols, "x"), _ptr(p, torch.float32, self.nrows, "p"),
+            _ptr(w, torch.float32, self.nrows, "w"), dptr, _ptr(f, torch.float64, 1, "f"),
+            _ptr(g, torch.float32, self.ncols, "g"), _raw_stream(stream))
+        if st:
+            _check(st)
         return (f, g, d) if want_d else (f, g)
 
     def pg_step(self, x, p, w, eta: float, f=None, g=None, stream=None):
@@ -450,11 +482,13 @@ class DoseMatrix:
         torch = _torch()
         if f is None:
             f = torch.empty(1, dtype=torch.float64, device=x.device)
-        gptr = _dptr(g, torch.float32, self.ncols, "g") if g is not None else None
-        _check(load().dose_pg_step(self._h, _dptr(x, torch.float32, self.ncols, "x"),
-                                   _dptr(p, torch.float32, self.nrows, "p"),
-                                   _dptr(w, torch.float32, self.nrows, "w"), ctypes.c_float(eta),
-                                   _dptr(f, torch.float64, 1, "f"), gptr, _stream_handle(stream)))
+        gptr = _ptr(g, torch.float32, self.ncols, "g") if g is not None else None
+        st = _fast().dose_pg_step(self._h, _ptr(x, torch.float32, self.ncols, "x"),
+                                  _ptr(p, torch.float32, self.nrows, "p"),
+                                  _ptr(w, torch.float32, self.nrows, "w"), ctypes.c_float(eta),
+                                  _ptr(f, torch.float64, 1, "f"), gptr, _raw_stream(stream))
+        if st:
+            _check(st)
         return f
 
     # ---- schedule
@@ -528,11 +562,11 @@ def spmv_batched(mats, Xs, Ds=None, stream=None):
     if Ds is None:
         Ds = [torch.empty((A.nrows, nvec), dtype=torch.float32, device=Xs[0].device) for A in mats]
     hs = (ctypes.c_void_p * n)(*[A.handle.value for A in mats])
-    xp = (ctypes.c_void_p * n)(*[_dptr(X, torch.float32, A.ncols * nvec, "X").value
-                                 for A, X in zip(mats, Xs)])
-    dp = (ctypes.c_void_p * n)(*[_dptr(D, torch.float32, A.nrows * nvec, "D").value
-                                 for A, D in zip(mats, Ds)])
-    _check(load().dose_spmv_batched(hs, n, xp, dp, nvec, _stream_handle(stream)))
+    xp = (ctypes.c_void_p * n)(*[_ptr(X, torch.float32, A.ncols * nvec, "X") for A, X in zip(mats, Xs)])
+    dp = (ctypes.c_void_p * n)(*[_ptr(D, torch.float32, A.nrows * nvec, "D") for A, D in zip(mats, Ds)])
+    st = _fast().dose_spmv_batched(hs, n, xp, dp, nvec, _raw_stream(stream))
+    if st:
+        _check(st)
     return Ds
 
 
@@ -567,12 +601,14 @@ class ScenarioSet:
         dev = x.device
         f = torch.empty(1, dtype=torch.float64, device=dev) if f is None else f
         g = torch.empty(self.ncols, dtype=torch.float32, device=dev) if g is None else g
-        _check(load().dose_robust_quadratic(
-            self._h, ROBUST_MODES[mode], _dptr(x, torch.float32, self.ncols, "x"),
-            _dptr(p, torch.float32, self.nrows, "p"), _dptr(w, torch.float32, self.nrows, "w"),
-            _dptr(f, torch.float64, 1, "f"),
-            _dptr(f_scen, torch.float64, len(self.mats), "f_scen") if f_scen is not None else None,
-            _dptr(g, torch.float32, self.ncols, "g"), _stream_handle(stream)))
+        st = _fast().dose_robust_quadratic(
+            self._h, ROBUST_MODES[mode], _ptr(x, torch.float32, self.ncols, "x"),
+            _ptr(p, torch.float32, self.nrows, "p"), _ptr(w, torch.float32, self.nrows, "w"),
+            _ptr(f, torch.float64, 1, "f"),
+            _ptr(f_scen, torch.float64, len(self.mats), "f_scen") if f_scen is not None else None,
+            _ptr(g, torch.float32, self.ncols, "g"), _raw_stream(stream))
+        if st:
+            _check(st)
         return (f, g, f_scen) if f_scen is not None else (f, g)
 
     def pg_step(self, x, p, w, eta: float, mode: str = "expected", f=None, g=None, stream=None):
@@ -609,11 +645,13 @@ def _autograd():
         @staticmethod
         def forward(ctx, x, A):
             ctx.A = A
-            return A.spmv(x.contiguous())
+            return A.spmv(x if x.is_contiguous() else x.contiguous())
 
         @staticmethod
         def backward(ctx, grad_d):
-            return ctx.A.adjoint(grad_d.contiguous().float()), None
+            if grad_d.dtype != torch.float32 or not grad_d.is_contiguous():
+                grad_d = grad_d.contiguous().float()
+            return ctx.A.adjoint(grad_d), None
 
     class _Quadratic(torch.autograd.Function):
         """f(x) = sum w (A x - p)^2 in one fused pass; backward scales the saved gradient."""
