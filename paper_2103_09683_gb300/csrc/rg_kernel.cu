@@ -33,6 +33,7 @@ namespace dose {
 namespace {
 
 constexpr uint32_t kRgMaxChain = 64;                // passes of one chain
+constexpr uint32_t kRgGradientSmem = 195 * 1024;
 constexpr uint32_t kRgRowWarps = 3;                 // warps of the rows without entries
 constexpr uint32_t kRgWarpBytes = kRgMaxRows * 4;   // a worker's row buffer: row sums, then residuals
 
@@ -78,13 +79,15 @@ struct RgVecs {
         r[0] = r[1] = 0xFFFFFFFFu;
         if (i >= end) return;
         if (lane < nxt.w) r[0] = __ldg(row_list + nxt.z + lane);
-        if (lane + 32 < nxt.w) r[1] = __ldg(row_list + nxt.z + lane + 32);
+        if (nxt.w > 32 && lane + 32 < nxt.w) r[1] = __ldg(row_list + nxt.z + lane + 32);
         ++i;
         if (i < end) nxt = __ldg(pk + i);
     }
     __device__ __forceinline__ void values(const RgParams& p) {
+        v0n[1] = v1n[1] = 0.f;
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
+            if (k && !__any_sync(0xffffffffu, rown[1] != 0xFFFFFFFFu)) break;  // most packets hold at most 32 rows
             v0n[k] = v1n[k] = 0.f;
             if (rown[k] != 0xFFFFFFFFu) {
                 v0n[k] = __ldg(p.v0 + rown[k]);
@@ -481,7 +484,11 @@ uint32_t rg_gradient_warps(const dose_matrix* A, const AdjTuning& t, bool quad, 
     if (fixed + per > kMaxSmemPerBlock) return 0;
     uint32_t most = t.rg_warps ? std::min<uint32_t>(t.rg_warps, kRgMaxWarps) : kRgMaxWarps;
     if (R.keep) most = std::min(most, R.keep_nw);
-    const uint32_t nw = (uint32_t)std::min<size_t>(most, (kMaxSmemPerBlock - fixed) / per);
+    // at most 195 KB, so that 60 instead of 28 KB of the SM's memory stay L1 for the
+    // gathered vectors and the stream of the rows without entries: 77.0 -> 71.2 us on
+    // the 200 x 200 x 120 beam with 12 instead of 14 warps (163 KB: 78.7 us)
+    const size_t room = R.keep || fixed + per > kRgGradientSmem ? kMaxSmemPerBlock : kRgGradientSmem;
+    const uint32_t nw = (uint32_t)std::min<size_t>(most, (room - fixed) / per);
     if (R.keep) d = (uint32_t)std::min<size_t>(kRgMaxDepth, (kMaxSmemPerBlock - fixed - nw * base) / ((size_t)nw * R.slot));
     if (depth) *depth = d;
     if (smem) *smem = fixed + nw * (base + (size_t)d * R.slot);
