@@ -65,41 +65,7 @@ inline RgView rg_view(const dose_matrix* A, int which) {
 
 #ifdef __CUDACC__
 
-// ---- packed FP32 pairs (f32x2): {lo, hi} in one 64-bit register; each half is
-// rounded as the scalar operation rounds.
 namespace dev {
-__device__ __forceinline__ uint64_t f2_splat(float a) {
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(a));
-    return r;
-}
-__device__ __forceinline__ uint64_t f2_pack(uint32_t lo, uint32_t hi) {
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(lo), "r"(hi));
-    return r;
-}
-__device__ __forceinline__ uint64_t f2_packf(float lo, float hi) {
-    return f2_pack(__float_as_uint(lo), __float_as_uint(hi));
-}
-__device__ __forceinline__ void f2_split(uint64_t v, float& lo, float& hi) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
-    uint64_t r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-
 // All bulk stores of this thread done (source read and data written).
 __device__ __forceinline__ void bulk_s2g(void* dst, const void* src, uint32_t bytes) {
     asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_u32(src)), "r"(bytes)
@@ -347,7 +313,7 @@ struct RgStream {
 // call is masked (its lanes past n read nothing and add 0 * the zero element).
 template <int FMT, int HR, uint32_t IW, int K>
 __device__ __forceinline__ void rg_dot_steps(const unsigned char* cols, const unsigned char* vals, uint32_t n,
-                                             uint32_t lane, const float* xs, uint32_t zc, uint64_t (&acc)[HR / 2]) {
+                                             uint32_t lane, const float* xs, uint32_t zc, uint64_t* acc) {
     RgVal<FMT, HR> q[K];
     uint32_t c[K];
 #pragma unroll
@@ -374,7 +340,7 @@ __device__ __forceinline__ void rg_dot_steps(const unsigned char* cols, const un
 
 template <int FMT, int HR, uint32_t IW>
 __device__ __forceinline__ void rg_dot(const unsigned char* cols, const unsigned char* vals, uint32_t n, uint32_t lane,
-                                       const float* xs, uint32_t zc, uint64_t (&acc)[HR / 2]) {
+                                       const float* xs, uint32_t zc, uint64_t* acc) {
     constexpr uint32_t VB = RgVal<FMT, HR>::kBytes;
     while (n > 128) {
         rg_dot_steps<FMT, HR, IW, 4>(cols, vals, 128, lane, xs, zc, acc);
@@ -391,7 +357,8 @@ __device__ __forceinline__ void rg_dot(const unsigned char* cols, const unsigned
 }
 
 // Totals over the warp of HR row sums (a transposed butterfly): lane l returns
-// row l / (32 / HR)'s total, the same value in all of that row's lanes.
+// row l / (32 / HR)'s total, the same value in all of that row's lanes.  Every
+// sum is the same tree (l with l ^ 16, then ^ 8, ^ 4, ^ 2, ^ 1) for any HR.
 template <int HR>
 __device__ __forceinline__ float rg_reduce(const uint64_t (&acc)[HR / 2], uint32_t lane) {
     float a[HR];

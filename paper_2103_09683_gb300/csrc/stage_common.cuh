@@ -641,6 +641,69 @@ __device__ __forceinline__ float dot_strided(const SlotView& v, uint32_t xs, uin
     return __fadd_rn(__fadd_rn(a0, a1), __fadd_rn(a2, a3));
 }
 
+// As dot_vec_p with compensated sums (Dot2): four accumulator pairs (s, c) as two
+// packed FP32 pairs each, so that one instruction does two entries' step of
+// TwoProduct and TwoSum (11 packed instructions per two entries).
+template <int FMT, uint32_t L, uint32_t IW>
+__device__ __forceinline__ void dot_vec_comp_p(const SlotPtrs<FMT, IW>& sp, const float* __restrict__ xsp, uint32_t zc,
+                                               uint32_t kb, uint32_t ke, uint32_t li, uint32_t iters, float& sum,
+                                               float& comp) {
+    const uint64_t m1 = dev::f2_splat(-1.0f);
+    uint64_t s[2] = {0ull, 0ull}, c[2] = {0ull, 0ull};
+    const int len = (int)(ke - kb);
+    const uint32_t kb4 = kb & ~3u;
+    int off = (int)(4 * li) - (int)(kb & 3u);
+    uint32_t k4 = kb4 + 4 * li;
+#pragma unroll 2
+    for (uint32_t it = 0; it < iters; ++it, off += 4 * L, k4 += 4 * L) {
+        const uint32_t kg = off < len ? k4 : kb4;
+        uint32_t j[4];
+        if (IW == 4) {
+            const uint4 cc = *reinterpret_cast<const uint4*>(static_cast<const uint32_t*>(sp.col) + kg);
+            j[0] = cc.x; j[1] = cc.y; j[2] = cc.z; j[3] = cc.w;
+        } else {
+            const uint2 cc = *reinterpret_cast<const uint2*>(static_cast<const uint16_t*>(sp.col) + kg);
+            j[0] = cc.x & 0xFFFFu; j[1] = cc.x >> 16; j[2] = cc.y & 0xFFFFu; j[3] = cc.y >> 16;
+        }
+        float a[4], x[4];
+        load_vals4<FMT>(sp.val + kg, a);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const bool m = (uint32_t)(off + u) < (uint32_t)len;
+            a[u] = m ? a[u] : 0.f;
+            x[u] = xsp[m ? j[u] : zc];
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const uint64_t av = dev::f2_packf(a[2 * h], a[2 * h + 1]), xv = dev::f2_packf(x[2 * h], x[2 * h + 1]);
+            const uint64_t np = dev::f2_mul(av, dev::f2_mul(xv, m1));  // -p, p = fl(a x)
+            const uint64_t e = dev::f2_fma(av, xv, np);                // a x - p
+            // TwoSum(s, p); a difference u - v is fma(v, -1, u), rounded as u - v is
+            const uint64_t t = dev::f2_fma(np, m1, s[h]);
+            const uint64_t bp = dev::f2_fma(s[h], m1, t);
+            const uint64_t as = dev::f2_fma(dev::f2_fma(bp, m1, t), m1, s[h]);
+            const uint64_t err = dev::f2_fma(dev::f2_add(np, bp), m1, as);
+            s[h] = t;
+            c[h] = dev::f2_add(c[h], dev::f2_add(err, e));
+        }
+    }
+    float sv[4], cv[4];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        dev::f2_split(s[h], sv[2 * h], sv[2 * h + 1]);
+        dev::f2_split(c[h], cv[2 * h], cv[2 * h + 1]);
+    }
+    sum = sv[0];
+    comp = cv[0];
+#pragma unroll
+    for (int u = 1; u < 4; ++u) {
+        float t, e;
+        dev::two_sum(sum, sv[u], t, e);
+        sum = t;
+        comp = __fadd_rn(__fadd_rn(comp, cv[u]), e);
+    }
+}
+
 // Compensated version (Dot2 of Ogita, Rump and Oishi, 2005): returns (s, c)
 // with s + c the dot product to about twice the working precision.
 template <int FMT, uint32_t IW = 4>
