@@ -869,7 +869,7 @@ static dose_status create_matrix(const dose_csr_desc* desc, unsigned flags, cons
         bool ok = build_row_groups(A.get(), A->rg, false, A->host_row_ptr.data(), col.data(), vals.data(), scl.data(), &why, &e);
         uint64_t full = 0;
         for (uint32_t i = 0; i < nrows; ++i) full += A->host_row_ptr[i + 1] > A->host_row_ptr[i];
-        if (ok && !A->rg.forward_only && (plan || full < kRgKeepRows) &&
+        if (ok && !A->rg.forward_only && full < (plan ? kRgKeepPlanRows : kRgKeepRows) &&
             !build_row_groups(A.get(), A->rgf, true, A->host_row_ptr.data(), col.data(), vals.data(), scl.data(), &why, &e)) {
             free_row_groups(A->rg);
             ok = false;

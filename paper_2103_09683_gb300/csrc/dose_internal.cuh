@@ -252,7 +252,7 @@ struct dose_matrix {
     dose::SellArrays sell;  // DOSE_CREATE_SELL only
 
     dose::RowGroups rg;     // row-group layout (when it applies)
-    dose::RowGroups rgf;    // ... in the stored-row order, for the fused pass (small matrices, multi-beam plans)
+    dose::RowGroups rgf;    // ... in the stored-row order, for the fused pass of small matrices
 
     // adjoint scratch: per-CTA partial gradients and objective values
     float* g_part = nullptr;     // adj.grid * ncols
@@ -380,8 +380,13 @@ constexpr uint32_t kRgDefaultUnion = 320;  // union columns of a packet (6 KB wi
 constexpr uint32_t kRgMaxRows = 64;        // rows of a packet
 constexpr uint32_t kRgZeroRun = 1024;      // rows of a run without entries
 // The fused pass keeps the stored-row order up to this many rows with entries (rg_layout.cu):
-// beyond, another order moves f by at most 4e-10 of itself (measured on beams of 0.5 to 7e5 rows)
-constexpr uint32_t kRgKeepRows = 200000;
+// beyond, another order moves f by at most 4e-10 of itself (measured on beams of 0.5 to 7e5
+// rows).  A plan of several beams has doses near the prescription and so an f of small
+// differences (moved by up to 3e-9 on 1.5e5 rows, 1.1e-9 on 8e5): it keeps the order longer.
+// Large plans do not, as it costs them more than half the step (nine scenarios of a 160 x
+// 160 x 100 plan, 8e5 rows: 2.30 ms in the kept order, 0.94 in the new one, 1.90 with the
+// stage-ring kernels).
+constexpr uint32_t kRgKeepRows = 200000, kRgKeepPlanRows = 400000;
 constexpr uint32_t kMaxAdjWarps = 20;      // producer + forward + scatter warps of the adjoint kernels
 constexpr uint32_t kSellDefaultSigma = 1u << 20;  // rows per sorting window of the SELL copy
 constexpr uint32_t kAdjMinScatterWarps = 8;
