@@ -255,8 +255,9 @@ dose_status dose_spmv(const dose_matrix* A, const float* x, float* d, void* stre
  * m <= n is the most terms any one accumulator of the row adds (a handful on the
  * default schedule) and g(m) = m 2^-24 / (1 - m 2^-24).  DOSE_SPMV_F64_NATIVE
  * accumulates with FP64 FMAs: |error| <= (n + 2) 2^-53 sum_k |a_ik x_k|.
- * Uses a handle-owned scratch copy of x (ncols + 1 doubles) and two launches on
- * `stream`; the same-stream rule for calls on one handle applies. */
+ * On the CSR arrays it uses a handle-owned scratch copy of x (ncols + 1 doubles)
+ * and two launches on `stream`, on row groups one launch; the same-stream rule for
+ * calls on one handle applies. */
 dose_status dose_spmv_f64(const dose_matrix* A, const double* x, double* d, unsigned flags, void* stream);
 
 /* D_m = A_m X_m for m < count, all in one persistent launch (one dose evaluation
@@ -378,7 +379,7 @@ dose_status dose_set_tuning(dose_matrix* A, const dose_tuning* tuning);
 /* Autotuner (the execution-configuration sweep of Sec. V-A, Fig. 4, for this
  * library's knobs).  Purposes: which calls the knobs are chosen for. */
 #define DOSE_TUNE_FORWARD 1u /* dose_spmv: stage tiles, lanes-per-row target, pipeline depth */
-#define DOSE_TUNE_FUSED 2u   /* dose_fwd_adj_quadratic / dose_pg_step with p = w = 1: adjoint layout
+#define DOSE_TUNE_FUSED 2u   /* dose_fwd_adj_quadratic / dose_pg_step with p = 0, w = 1: adjoint layout
                                 (row groups or CSR) and its tiles and warps */
 #define DOSE_TUNE_BATCHED 4u /* dose_spmv_batched of this matrix with 16 vectors (same knobs as
                                 DOSE_TUNE_FUSED; with both, their summed time is minimised) */

@@ -451,7 +451,8 @@ dose_status sweep(dose_matrix* A, const float* x, unsigned purposes, cudaStream_
         x = S.x1;
     }
     if (e == cudaSuccess) e = dev_malloc(&S.d, nr * 4);
-    if (e == cudaSuccess) e = upload_fill(&S.pw, 2 * nrp, 1.0f);  // p = 1, w = 1 on every row
+    if (e == cudaSuccess) e = upload_fill(&S.pw, 2 * nrp, 1.0f);
+    if (e == cudaSuccess) e = cudaMemset(S.pw, 0, nrp * 4);  // p = 0 (as outside a target), w = 1 on every row
     if (e == cudaSuccess) e = dev_malloc(&S.g, nc * 4);
     if (e == cudaSuccess) e = dev_malloc(&S.f, 8);
     if (e == cudaSuccess) e = cudaEventCreate(&S.e0);
@@ -529,8 +530,8 @@ dose_status sweep(dose_matrix* A, const float* x, unsigned purposes, cudaStream_
         ms[0] = m;
     }
 
-    // 2. the fused objective pass (p = w = 1 on every row, so the objective
-    //    terms of rows without entries are paid as in use) and the batched SpMM:
+    // 2. the fused objective pass (p = 0 and w = 1 on every row: what rows without
+    //    entries cost in use, where nothing is prescribed) and the batched SpMM:
     //    the adjoint layout and its knobs, scored by the sum of their times
     if (purposes & (DOSE_TUNE_FUSED | DOSE_TUNE_BATCHED)) {
         const bool time_b = (purposes & DOSE_TUNE_BATCHED) && S.X16;
