@@ -46,9 +46,13 @@ uint32_t round_up16(uint32_t v) { return (v + 15) / 16 * 16; }
 constexpr uint32_t kMaxRowEntries = 4096;  // longest row of the gradient passes (and most columns of a packet)
 constexpr uint32_t kMaxForwardRow = 32768; // ... of a layout for the forward passes alone
 constexpr uint32_t kTile = 8;              // voxels per side of the tiles the rows are ordered by
-constexpr uint64_t kGroupCost = 4;         // dealing cost of a group, in steps of 32 columns: its reduction,
-                                           // outputs and its share of its packet (140 instructions against
-                                           // 21 a step in dose_spmv, 280 against 44 in the fused pass)
+// Dealing cost of a group, in steps of 32 columns: its reduction, outputs and its share
+// of its packet.  By instructions it is 7 steps in dose_spmv (140 against 21 a step) and 6
+// in the fused pass, less with FP64 or 16 vectors, whose steps are longer.  Measured with
+// costs of 4 / 3 / 2: dose on 1.5e8 entries 66.7 / 66.3 / 66.5 us, fused pass on 6.3e7
+// entries 71.2 / 71.7 / 72.9, FP64 dose 62.2 / 60.6 / 58.2, three matrices times 16 vectors
+// 142.5 / 138.4 / 137.7.  3 gives the FP64 and batched forms most of their gain.
+constexpr uint64_t kGroupCost = 3;
 
 cudaError_t rg_upload(void** dst, const void* src, size_t bytes, size_t alloc_bytes) {
     alloc_bytes = std::max<size_t>(alloc_bytes, 16);
@@ -373,7 +377,7 @@ struct Grp {
 // added; a projected-gradient loop carries them on from step to step.  Over many
 // rows such differences average out (2e-10 of f over 2.5e5 rows), over few they
 // do not (up to 3e-9 on small plans, 1e-8 after 100 steps).  So the fused pass of
-// small matrices and of multi-beam plans keeps one fixed order, whatever order
+// small matrices (kRgKeepRows, kRgKeepPlanRows) keeps one fixed order, whatever order
 // the other passes' groups take: groups of up to four consecutive non-empty rows,
 // cut into stages of consecutive groups, stages dealt to CTAs by column windows
 // and the groups of a stage dealt round-robin to the warps, a step further at
