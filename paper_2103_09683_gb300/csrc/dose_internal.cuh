@@ -382,7 +382,7 @@ constexpr uint32_t kRgZeroRun = 1024;      // rows of a run without entries
 // The fused pass keeps the stored-row order up to this many rows with entries (rg_layout.cu):
 // beyond, another order moves f by at most 4e-10 of itself (measured on beams of 0.5 to 7e5
 // rows).  A plan of several beams has doses near the prescription and so an f of small
-// differences (moved by up to 3e-9 on 1.5e5 rows, 1.1e-9 on 8e5): it keeps the order longer.
+// differences (moved by up to 3e-9 on 1.5e5 rows, 1.4e-9 on 4e5 to 8e5): it keeps the order longer.
 // Large plans do not, as it costs them more than half the step (nine scenarios of a 160 x
 // 160 x 100 plan, 8e5 rows: 2.30 ms in the kept order, 0.94 in the new one, 1.90 with the
 // stage-ring kernels).

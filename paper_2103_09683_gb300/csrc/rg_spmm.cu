@@ -41,6 +41,11 @@ struct FwdParams {
     int* err;
 };
 
+// Bound by memory and issue alike: 1.5e8 entries (u16, 16-bit columns, 408 MB of its
+// own bytes) take 66.3 us, 0.90 of 6.8 TB/s, against 109.6 us with groups of four
+// consecutive rows (488 MB, 0.66) and one ring of stages for all warps of a CTA: eight
+// rows share each column and each x, so a third of the instructions went, and a warp
+// never waits for the others' packets.
 template <int FMT, int HR, uint32_t IW>
 __global__ void __launch_bounds__((kMvWorkers + 1) * 32, 1) rg_spmv_kernel(const __grid_constant__ FwdParams p) {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -200,6 +205,10 @@ struct Acc64<F64_DP, HR> {
     }
 };
 
+// Bound by the FP32 pair arithmetic (issue 63 % active, memory 42 %), so one packed
+// instruction does two rows' step: 6.3e7 F16 entries take 60.0 us, against 111.5 us
+// entry by entry on CSR (twice the instructions and 2.5 times the bytes).  16 warps:
+// the pairs of eight rows take 94 registers a thread.
 template <int FMT, int HR, uint32_t IW, int MODE>
 __global__ void __launch_bounds__((kMv64Workers + 1) * 32, 1) rg_spmv64_kernel(const __grid_constant__ FwdParams p) {
     constexpr uint32_t VB = RgVal<FMT, HR>::kBytes;
@@ -296,6 +305,11 @@ __device__ __forceinline__ uint32_t mm_x(uint32_t c, uint32_t q) {
 // and 2 HR packed FMAs (rows 2 i and 2 i + 1 times one vector's weight).  NQ =
 // quads of vectors (1, 2 or 4): fewer vectors put more lanes on the columns
 // instead of computing vectors nobody asked for.
+// Bound by issue (47 % active) and the spread of the CTAs' times (mean 84 % of the
+// longest): 16 vectors times three matrices (160 x 160 x 80 voxels, 1000 spots) take
+// 138.4 us, 172.9 with groups of four rows, whose X loads were twice as many and kept
+// the shared memory 56 % busy (33 % now); 5 vectors times two matrices 36.6 us, 96.9
+// when 16 were always computed.  12 warps: 96 registers a thread.
 template <int FMT, int HR, uint32_t IW, int NQ>
 __global__ void __launch_bounds__((kMmWorkers[0] + 1) * 32, 1) rg_spmm_kernel(const __grid_constant__ MmParams p) {
     constexpr uint32_t VB = RgVal<FMT, HR>::kBytes;
