@@ -161,11 +161,14 @@ typedef struct {
        CSR forms.  A non-finite x_j or residual reaches every row of a group whose union
        holds column j (0 * inf), not only the rows that store j. */
     uint32_t adj_layout;
-    uint32_t rg_tile_union;     /* row groups: most union columns per packet (what one warp copies at a
-                                   time; 256..8192, at most 320 are used; default 320).  Packets are cut
-                                   at create; a later value is checked and reported only.  It must not
-                                   be smaller than the longest row. */
-    uint32_t rg_tile_rows;      /* row groups: checked and reported (256..8192); a packet holds at most 64 rows */
+    uint32_t rg_tile_union;     /* row groups: union columns a warp copies at a time (256..8192, at least the
+                                   longest row where that is at most 4096; at most 320 are used).  Packets are
+                                   cut at create; a later value is checked and reported only.  Where the
+                                   fused pass keeps the stored-row order (see rg_groups in dose_info), also
+                                   the union columns of one stage of that order.  Default by format (2048 to
+                                   6816), at least the longest row. */
+    uint32_t rg_tile_rows;      /* row groups: rows a stage of the stored-row order spans, at create (256..8192;
+                                   default 512); a packet holds at most 64 rows */
     uint32_t rg_stages;         /* row groups: packets in flight per warp of the adjoint and fused passes
                                    (2..8; at most 4 are used; default 2) */
     uint32_t rg_warps;          /* row groups: worker warps of those passes (1..15; 0 = as many as fit) */

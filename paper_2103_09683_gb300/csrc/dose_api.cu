@@ -1231,16 +1231,17 @@ dose_status dose_set_tuning(dose_matrix* A, const dose_tuning* tuning) {
     dose_status st = check_tuning(A, t);
     if (st == DOSE_OK) st = check_adj_tuning(at);
     if (st != DOSE_OK) return st;
-    cudaError_t e = cudaDeviceSynchronize();
-    if (e != cudaSuccess) return cuda_fail(e, "dose_set_tuning");
-    st = apply_schedule(A, A->fwd, t, A->fwd_windowed);
-    if (st == DOSE_OK && A->fwd64_own) st = apply_schedule(A, A->fwd64, t, false);
-    if (st != DOSE_OK) return st;
+    // everything is checked before any schedule is cut anew
     if (at.layout == 2 && (!A->rg.built || A->rg.forward_only)) return invalid("adj_layout = 2: the handle has no row-group layout");
     if (t.layout == 2 && (!A->rg.built || A->rg.forward_only || (A->flags & DOSE_CREATE_COMPENSATED)))
         return invalid("fwd_layout = 2: dose_spmv cannot run on the row-group layout of this handle");
     if (A->rg.built && !A->rg.forward_only && at.rg_tile_u != A->adj_tuning.rg_tile_u && A->max_row_len > at.rg_tile_u)
         return invalid("tuning.rg_tile_union is smaller than the longest row");
+    cudaError_t e = cudaDeviceSynchronize();
+    if (e != cudaSuccess) return cuda_fail(e, "dose_set_tuning");
+    st = apply_schedule(A, A->fwd, t, A->fwd_windowed);
+    if (st == DOSE_OK && A->fwd64_own) st = apply_schedule(A, A->fwd64, t, false);
+    if (st != DOSE_OK) return st;
     A->adj_tuning = at;
     if (A->rg.built && (e = rg_schedule(A)) != cudaSuccess) return cuda_fail(e, "row-group schedule");
     return apply_schedule(A, A->adj, adj_schedule_tuning(t, at), true);

@@ -191,7 +191,7 @@ struct RowGroups {
     RgDeal deal[RG_DEALS];
     uint32_t wmax = 0;              // most columns of any CTA
     uint32_t slot = 0;              // bytes of a ring slot (the largest packet)
-    uint32_t tile_u = 0;            // union columns per packet asked for
+    uint32_t tile_u = 0;            // rg_tile_union in effect (0: rows past the gradient passes' limit, none given)
     uint64_t data_bytes = 0;        // of the packets
     uint64_t bytes = 0;             // device bytes of the arrays above
     std::vector<uint4> host_pk;     // the packets in memory order, as in RgDeal
@@ -212,7 +212,7 @@ struct AdjTuning {
     // layout of the adjoint / fused passes: 0 = row groups where they apply, else
     // CSR; 1 = CSR; 2 = row groups (create fails if they do not apply)
     uint32_t layout = 0;
-    uint32_t rg_tile_u = 0;        // row groups: union columns per packet, at create (0 = kRgDefaultUnion)
+    uint32_t rg_tile_u = 0;        // row groups: union columns, at create (0 = default_tile_u, rg_layout.cu)
     uint32_t rg_tile_rows = 512;   // row groups: accepted and reported; packets hold at most kRgMaxRows rows
     uint32_t rg_stages = 2;        // row groups: slots of a gradient warp's ring
     uint32_t rg_warps = 0;         // row groups: gradient warps (0 = as many as fit, up to kRgMaxWarps)

@@ -54,6 +54,14 @@ constexpr uint32_t kTile = 8;              // voxels per side of the tiles the r
 // 142.5 / 138.4 / 137.7.  3 gives the FP64 and batched forms most of their gain.
 constexpr uint64_t kGroupCost = 3;
 
+// rg_tile_union where the caller gave none: about 40 KB of union columns and values
+// (a stage of the stored-row order, below), never less than the longest row, so that
+// the reported value can be given back.
+uint32_t default_tile_u(uint32_t max_row_len, uint32_t iw, uint32_t es) {
+    const uint32_t def = std::max(512u, std::min(8192u, 40960 / (iw + 4 * es) / 32 * 32));
+    return std::max(def, (max_row_len + 31) / 32 * 32);
+}
+
 cudaError_t rg_upload(void** dst, const void* src, size_t bytes, size_t alloc_bytes) {
     alloc_bytes = std::max<size_t>(alloc_bytes, 16);
     cudaError_t e = dev_malloc(dst, alloc_bytes);
@@ -809,7 +817,8 @@ bool build_row_groups(dose_matrix* A, RowGroups& R, bool keep, const uint32_t* r
         *why = too_long;
         return false;
     }
-    const uint32_t tile_u = A->adj_tuning.rg_tile_u ? A->adj_tuning.rg_tile_u : kRgDefaultUnion;
+    const uint32_t tile_u =
+        A->adj_tuning.rg_tile_u ? A->adj_tuning.rg_tile_u : forward_only ? 0u : default_tile_u(A->max_row_len, R.iw, es);
     if (A->max_row_len > tile_u && A->adj_tuning.rg_tile_u && !forward_only) {
         *err = cudaErrorInvalidValue;
         return false;
@@ -823,7 +832,7 @@ bool build_row_groups(dose_matrix* A, RowGroups& R, bool keep, const uint32_t* r
         const uint32_t* cmin = A->host_row_cmin.data();
         const uint32_t* cmax = A->host_row_cmax.data();
         // columns a packet may hold: the slot of a warp is a few KB
-        const uint32_t cap = std::min(tile_u, kRgDefaultUnion);
+        const uint32_t cap = tile_u ? std::min(tile_u, kRgDefaultUnion) : kRgDefaultUnion;
         uint32_t max_u = cap;
         std::vector<std::vector<Grp>> sg;
         std::vector<std::vector<uint32_t>> su;
@@ -839,16 +848,12 @@ bool build_row_groups(dose_matrix* A, RowGroups& R, bool keep, const uint32_t* r
                 su[0].insert(su[0].end(), u.begin(), u.end());
             });
             const AdjTuning& t = A->adj_tuning;
-            uint32_t nu_max = 0;
-            for (const Grp& g : sg[0]) nu_max = std::max(nu_max, g.nu);
-            const uint32_t def = std::max(512u, std::min(8192u, 40960 / (R.iw + 4 * es) / 32 * 32));
-            const uint32_t tu = t.rg_tile_u ? t.rg_tile_u : std::max(def, (nu_max + 31) / 32 * 32);
-            KS = kept_schedule(M, rows, sg[0], su[0], R.iw, grid, tu, t.rg_tile_rows, M.scales != nullptr);
+            KS = kept_schedule(M, rows, sg[0], su[0], R.iw, grid, tile_u, t.rg_tile_rows, M.scales != nullptr);
             // the warps that fitted beside this order's stages and windows; packets as
             // large as two slots each leave room for
             auto r128 = [](uint64_t v) { return (v + 127) / 128 * 128; };
             const uint64_t own = r128(4ull * KS.wwidth), most = t.rg_warps ? std::min<uint32_t>(t.rg_warps, kRgMaxWarps) : kRgMaxWarps;
-            const uint64_t stage = 128 + r128(kKeepStageGroups * 16) + r128((tu + 16) * R.iw) + r128((tu + 8ull) * 4 * es) +
+            const uint64_t stage = 128 + r128(kKeepStageGroups * 16) + r128((tile_u + 16) * R.iw) + r128((tile_u + 8ull) * 4 * es) +
                                    (M.scales ? 3 : 2) * r128((t.rg_tile_rows + 8) * 4);
             const uint64_t rest = 3072 + r128(4ull * KS.wwidth + 4) + t.rg_stages * stage;
             R.keep_nw = (uint32_t)(rest + own <= kMaxSmemPerBlock ? std::min<uint64_t>(most, (kMaxSmemPerBlock - rest) / own) : most);
