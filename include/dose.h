@@ -210,6 +210,10 @@ typedef struct {
     dose_tuning tuning;         /* the knobs in effect */
     uint32_t adj_layout_fused;  /* layout the fused pass runs on: 1 = CSR, 2 = row groups, 0 = none fits */
     uint32_t adj_layout_adjoint;/* ... dose_adjoint */
+    /* The four rg_* counts below are those of the layout that dose_spmv, the batched SpMM
+       and dose_adjoint run on.  The fused pass of small matrices (fewer than 200,000 rows
+       with entries; 400,000 for plans of several beams) runs on a second copy in the
+       stored-row order, four consecutive rows a group, which keeps the digits of f. */
     uint64_t rg_groups;         /* row groups built (0: the layout was not built) */
     uint64_t rg_union_entries;  /* values stored by the row groups / 4 (union columns x rows per group / 4) */
     uint32_t rg_window;         /* most columns any CTA sees on the row-group layout */

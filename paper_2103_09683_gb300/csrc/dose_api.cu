@@ -1210,7 +1210,7 @@ dose_status dose_matrix_info(const dose_matrix* A, dose_info* out) {
         out->rg_warps_fused = rg_gradient_warps(A, A->adj_tuning, true, nullptr, nullptr);
         if (rg_active(A, true)) {
             out->adj_layout_fused = 2;
-            out->adj_block_fused = 32 * out->rg_warps_fused;
+            out->adj_block_fused = 32 * (out->rg_warps_fused + kRgRowWarps);
             out->fused_bytes = rg_fused_bytes(A, false);
         }
         if (rg_active(A, false)) {

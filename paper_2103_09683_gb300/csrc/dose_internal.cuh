@@ -376,6 +376,7 @@ __host__ __device__ constexpr uint32_t value_bytes(int fmt) {
 }
 // Row-group layout: worker warps of the gradient kernels (one producer-less CTA per SM).
 constexpr uint32_t kRgMaxWarps = 15;
+constexpr uint32_t kRgRowWarps = 3;        // more warps of the fused pass, for the rows without entries
 constexpr uint32_t kRgDefaultUnion = 320;  // union columns of a packet (6 KB with eight 16-bit values each)
 constexpr uint32_t kRgMaxRows = 64;        // rows of a packet
 constexpr uint32_t kRgZeroRun = 1024;      // rows of a run without entries

@@ -34,7 +34,6 @@ namespace {
 
 constexpr uint32_t kRgMaxChain = 64;                // passes of one chain
 constexpr uint32_t kRgGradientSmem = 195 * 1024;
-constexpr uint32_t kRgRowWarps = 3;                 // warps of the rows without entries
 constexpr uint32_t kRgWarpBytes = kRgMaxRows * 4;   // a worker's row buffer: row sums, then residuals
 
 struct RgParams {

@@ -83,3 +83,12 @@ def test_a_refused_value_changes_nothing():
     with pytest.raises(dose.DoseError) as ei:
         make(csr, "u16", tuning=dict(rg_tile_union=512, adj_layout=2))
     assert ei.value.status == 1
+
+
+def test_reported_threads_per_cta():
+    """adj_block_*: every warp of the launch, those of the rows without entries too."""
+    for csr in (_long_rows(), dosegen.generate(dosegen.TINY)):
+        A, _ = make(csr, "u16", tuning=dict(rg_warps=5))
+        info = A.info()
+        assert info["rg_warps_fused"] == 5
+        assert info["adj_block_fused"] == 32 * (5 + 3) and info["adj_block_adjoint"] == 32 * 5
