@@ -871,8 +871,15 @@ static dose_status create_matrix(const dose_csr_desc* desc, unsigned flags, cons
         for (uint32_t i = 0; i < nrows; ++i) full += A->host_row_ptr[i + 1] > A->host_row_ptr[i];
         if (ok && !A->rg.forward_only && full < (plan ? kRgKeepPlanRows : kRgKeepRows) &&
             !build_row_groups(A.get(), A->rgf, true, A->host_row_ptr.data(), col.data(), vals.data(), scl.data(), &why, &e)) {
-            free_row_groups(A->rg);
-            ok = false;
+            // without room for the fused pass's own copy it runs on the other calls' layout
+            free_row_groups(A->rgf);
+            if (e == cudaErrorMemoryAllocation && A->adj_tuning.layout != 2) {
+                cudaGetLastError();
+                e = cudaSuccess;
+            } else {
+                free_row_groups(A->rg);
+                ok = false;
+            }
         }
         if (!ok && e == cudaErrorInvalidValue) {
             why = "tuning.rg_tile_union is smaller than the longest row";
@@ -889,6 +896,11 @@ static dose_status create_matrix(const dose_csr_desc* desc, unsigned flags, cons
         }
         if (ok) {
             e = rg_schedule(A.get());
+            if (e == cudaErrorMemoryAllocation && A->adj_tuning.layout != 2 && A->rgf.built) {
+                cudaGetLastError();
+                free_row_groups(A->rgf);
+                e = rg_schedule(A.get());
+            }
             if (e == cudaErrorMemoryAllocation && A->adj_tuning.layout != 2) {
                 cudaGetLastError();
                 free_row_groups(A->rg);

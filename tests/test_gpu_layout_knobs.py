@@ -6,8 +6,9 @@ import pytest
 import torch
 
 import dosegen
+import oracle
 import paper_2103_09683_gb300 as dose
-from gpu_helpers import make
+from gpu_helpers import adj_check, fwd_check, make
 
 pytestmark = pytest.mark.gpu
 
@@ -92,3 +93,36 @@ def test_reported_threads_per_cta():
         info = A.info()
         assert info["rg_warps_fused"] == 5
         assert info["adj_block_fused"] == 32 * (5 + 3) and info["adj_block_adjoint"] == 32 * 5
+
+
+def test_no_memory_for_the_fused_copy_keeps_the_layout(monkeypatch):
+    """Rows i, i + 64, ... see the same 25 columns, neighbours see others: the layout of
+    the other calls stores 2.25 bytes an entry, the stored-row copy of the fused
+    pass 10, the CSR columns 4.  With room for one more array of the columns' size the
+    layout stays, and the fused pass runs on it."""
+    n = 16000
+    base = np.random.default_rng(5).permutation(1600).reshape(64, 25)
+    base.sort(axis=1)
+    col = base[np.arange(n) % 64].astype(np.uint32).reshape(-1)
+    rp = (25 * np.arange(n + 1)).astype(np.uint32)
+    csr = dosegen.CSR(n, 1600, rp, col, np.random.default_rng(6).uniform(0.1, 1.0, col.size))
+    monkeypatch.setenv("DOSE_TEST_ALLOC_LIMIT", str(4 * ((csr.nnz + 3) // 4 * 4 + 16)))
+    with pytest.raises(dose.DoseError) as ei:
+        make(csr, "u16", tuning=dict(adj_layout=2))
+    assert ei.value.status == 2
+    A, enc = make(csr, "u16")
+    monkeypatch.delenv("DOSE_TEST_ALLOC_LIMIT")
+    info = A.info()
+    assert info["rg_groups"] > 0 and info["spmv_layout"] == 2
+    assert info["adj_layout_adjoint"] == 2 and info["adj_layout_fused"] == 2
+    rng = np.random.default_rng(7)
+    x = rng.uniform(0, 1, 1600).astype(np.float32)
+    p = rng.uniform(0, 2, n).astype(np.float32)
+    w = rng.uniform(0.5, 2.0, n).astype(np.float32)
+    f, g, d = A.fwd_adj_quadratic(_to(x), _to(p), _to(w), want_d=True)
+    fwd_check(d.cpu().numpy(), oracle.spmv(n, rp, col, enc.decoded, x))
+    f_own, r_own = oracle.objective(d.cpu().numpy().astype(np.float64), p, w)
+    assert abs(float(f.item()) - f_own) <= 1e-12 * f_own
+    adj_check(g.cpu().numpy(), oracle.spmv_t(n, 1600, rp, col, enc.decoded, r_own),
+              oracle.abs_spmv_t(n, 1600, rp, col, enc.decoded, r_own))
+    A.device_status()
