@@ -572,18 +572,11 @@ dose_status sweep(dose_matrix* A, const float* x, unsigned purposes, cudaStream_
                 *usable = false;
                 return DOSE_OK;
             }
-            if (a.tile_nnz != csr_cut.tile_nnz || a.tile_rows != csr_cut.tile_rows || a.stages != csr_cut.stages ||
-                a.row_order != csr_cut.row_order) {
-                const dose_status s2 = apply_schedule(A, A->adj, adj_schedule_tuning(A->fwd.tuning, a), true);
-                if (s2 != DOSE_OK) return s2;
-                csr_cut = a;
-            }
-            A->adj_tuning = a;
-            if (A->rg.built) {
-                const cudaError_t e2 = rg_schedule(A);
-                if (e2 != cudaSuccess) return cuda_fail(e2, "row-group schedule");
-            }
-            return DOSE_OK;
+            const bool recut = a.tile_nnz != csr_cut.tile_nnz || a.tile_rows != csr_cut.tile_rows ||
+                               a.stages != csr_cut.stages || a.row_order != csr_cut.row_order;
+            const dose_status s2 = apply_adj_knobs(A, A->fwd.tuning, a, recut);
+            if (s2 == DOSE_OK && recut) csr_cut = a;
+            return s2;
         };
         float best = 3e38f;
         AdjTuning best_a = base;

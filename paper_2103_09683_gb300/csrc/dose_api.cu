@@ -523,35 +523,51 @@ static cudaError_t upload(T** dst, const T* src, size_t n, size_t alloc_n) {
     return e;
 }
 
-// Build one schedule on the host and replace `D` with its device copy.  The
-// adjoint schedule (`windowed`) gets per-CTA column windows.
-dose_status apply_schedule(dose_matrix* A, DevSchedule& D, const Tuning& t, bool windowed) {
+// Build one schedule on the host and its device copy.  The adjoint schedule
+// (`windowed`) gets per-CTA column windows.  On an error nothing is left allocated.
+static dose_status make_schedule(const dose_matrix* A, uint32_t grid, const Tuning& t, bool windowed, DevSchedule* out) {
+    DevSchedule& D = *out;
+    D.grid = grid;
     const bool win = windowed && !A->host_row_cmin.empty();
     const uint32_t vbytes = value_bytes(A->fmt) + 4;
-    Schedule S = build_schedule(A->host_row_ptr, A->nrows, t, D.grid, win ? A->host_row_cmin.data() : nullptr,
+    Schedule S = build_schedule(A->host_row_ptr, A->nrows, t, grid, win ? A->host_row_cmin.data() : nullptr,
                                 win ? A->host_row_cmax.data() : nullptr, A->ncols, vbytes);
     if (win) {
         // Cutting blocks at every doubling of their column range narrows the
         // windows of a single beam (one more scatter warp fits on the clinical
         // beam) but only fragments a multi-beam plan, whose rows already span
         // every beam: keep it where it narrows the window.
-        Schedule T = build_schedule(A->host_row_ptr, A->nrows, t, D.grid, A->host_row_cmin.data(),
+        Schedule T = build_schedule(A->host_row_ptr, A->nrows, t, grid, A->host_row_cmin.data(),
                                     A->host_row_cmax.data(), A->ncols, vbytes, true);
         if (T.wwidth < S.wwidth) S = std::move(T);
     }
-    free_dev_schedule(D);
     cudaError_t e;
     if ((e = upload(&D.desc, S.desc.data(), S.desc.size(), S.desc.size() + 1)) != cudaSuccess ||
         (e = upload(&D.ne, S.ne.data(), S.ne.size(), (S.ne.size() + 7) / 8 * 8 + 16)) != cudaSuccess ||
         (e = upload(&D.cta_begin, S.cta_begin.data(), S.cta_begin.size(), S.cta_begin.size())) != cudaSuccess ||
-        (e = upload(&D.wlo, S.wlo.data(), S.wlo.size(), S.wlo.size())) != cudaSuccess)
+        (e = upload(&D.wlo, S.wlo.data(), S.wlo.size(), S.wlo.size())) != cudaSuccess) {
+        free_dev_schedule(D);
         return cuda_fail(e, "uploading the schedule");
+    }
     D.wwidth = S.wwidth;
     D.n_stages = (uint32_t)S.desc.size();
     D.n_coop_rows = S.n_coop_rows;
     std::memcpy(D.lanes_hist, S.lanes_hist, sizeof(D.lanes_hist));
     D.tuning = t;
     return DOSE_OK;
+}
+
+static void replace_schedule(DevSchedule& D, const DevSchedule& by) {
+    free_dev_schedule(D);
+    D = by;
+}
+
+// Replace `D` with the schedule of the knobs t; on an error D stays.
+dose_status apply_schedule(dose_matrix* A, DevSchedule& D, const Tuning& t, bool windowed) {
+    DevSchedule N;
+    const dose_status st = make_schedule(A, D.grid, t, windowed, &N);
+    if (st == DOSE_OK) replace_schedule(D, N);
+    return st;
 }
 
 // The adjoint schedule: its own tile sizes, the forward's lane binning.
@@ -563,6 +579,23 @@ Tuning adj_schedule_tuning(const Tuning& fwd, const AdjTuning& a) {
     t.stages = a.stages;
     t.row_order = a.row_order;
     return t;
+}
+
+// The gradient knobs a: the CSR schedule (cut anew if `recut`), the deals of the row
+// groups and adj_tuning together; on an error all of them stay.
+dose_status apply_adj_knobs(dose_matrix* A, const Tuning& fwd, const AdjTuning& a, bool recut) {
+    DevSchedule N;
+    if (recut) {
+        const dose_status st = make_schedule(A, A->adj.grid, adj_schedule_tuning(fwd, a), true, &N);
+        if (st != DOSE_OK) return st;
+    }
+    const cudaError_t e = rg_schedule(A, a);
+    if (e != cudaSuccess) {
+        free_dev_schedule(N);
+        return cuda_fail(e, "row-group schedule");
+    }
+    if (recut) replace_schedule(A->adj, N);
+    return DOSE_OK;
 }
 
 static uint64_t schedule_bytes(const DevSchedule& D) {
@@ -895,11 +928,11 @@ static dose_status create_matrix(const dose_csr_desc* desc, unsigned flags, cons
             why = "its arrays do not fit in device memory";
         }
         if (ok) {
-            e = rg_schedule(A.get());
+            e = rg_schedule(A.get(), A->adj_tuning);
             if (e == cudaErrorMemoryAllocation && A->adj_tuning.layout != 2 && A->rgf.built) {
                 cudaGetLastError();
                 free_row_groups(A->rgf);
-                e = rg_schedule(A.get());
+                e = rg_schedule(A.get(), A->adj_tuning);
             }
             if (e == cudaErrorMemoryAllocation && A->adj_tuning.layout != 2) {
                 cudaGetLastError();
@@ -1251,12 +1284,18 @@ dose_status dose_set_tuning(dose_matrix* A, const dose_tuning* tuning) {
         return invalid("tuning.rg_tile_union is smaller than the longest row");
     cudaError_t e = cudaDeviceSynchronize();
     if (e != cudaSuccess) return cuda_fail(e, "dose_set_tuning");
-    st = apply_schedule(A, A->fwd, t, A->fwd_windowed);
-    if (st == DOSE_OK && A->fwd64_own) st = apply_schedule(A, A->fwd64, t, false);
-    if (st != DOSE_OK) return st;
-    A->adj_tuning = at;
-    if (A->rg.built && (e = rg_schedule(A)) != cudaSuccess) return cuda_fail(e, "row-group schedule");
-    return apply_schedule(A, A->adj, adj_schedule_tuning(t, at), true);
+    DevSchedule fwd, fwd64;
+    st = make_schedule(A, A->fwd.grid, t, A->fwd_windowed, &fwd);
+    if (st == DOSE_OK && A->fwd64_own) st = make_schedule(A, A->fwd64.grid, t, false, &fwd64);
+    if (st == DOSE_OK) st = apply_adj_knobs(A, t, at, true);
+    if (st != DOSE_OK) {
+        free_dev_schedule(fwd);
+        free_dev_schedule(fwd64);
+        return st;
+    }
+    replace_schedule(A->fwd, fwd);
+    if (A->fwd64_own) replace_schedule(A->fwd64, fwd64);
+    return DOSE_OK;
 }
 
 dose_status dose_device_status(const dose_matrix* A, void* stream) {

@@ -307,11 +307,11 @@ dose_status adjoint_supported(const dose_matrix* A, bool quad, const float* cons
 // Row-group layout (rg_layout.cu).  build_row_groups forms the layout from the
 // host CSR and the stored values; false (with *why) if some row is too long
 // (*err = cudaErrorInvalidValue: longer than the caller's rg_tile_union), or with
-// *err set if memory ran out.  rg_schedule deals the packets to the warps of
-// each call (re-run when the tuning changes).
+// *err set if memory ran out.  rg_schedule makes t the gradient knobs
+// in effect and deals the packets to the warps of each call; on an error nothing changes.
 bool build_row_groups(dose_matrix* A, RowGroups& R, bool keep, const uint32_t* rp, const uint32_t* col,
                       const unsigned char* vals, const float* scales, std::string* why, cudaError_t* err);
-cudaError_t rg_schedule(dose_matrix* A);
+cudaError_t rg_schedule(dose_matrix* A, const AdjTuning& t);
 void free_row_groups(RowGroups& R);
 const RowGroups& rg_of(const dose_matrix* A, int which);  // the layout call RG_DEAL_* runs on
 // Worker warps of a call (RG_DEAL_*) that fit beside their slots, the depth of
@@ -363,6 +363,7 @@ dose_status check_adj_tuning(const AdjTuning& t);
 void merge_tuning(Tuning& t, AdjTuning& a, const dose_tuning* in);
 void export_tuning(const Tuning& t, const AdjTuning& a, dose_tuning* out);
 dose_status apply_schedule(dose_matrix* A, DevSchedule& D, const Tuning& t, bool windowed = false);
+dose_status apply_adj_knobs(dose_matrix* A, const Tuning& fwd, const AdjTuning& a, bool recut);
 Tuning adj_schedule_tuning(const Tuning& fwd, const AdjTuning& a);
 // FNV-1a of the matrix's shape, format, creation flags, row pointers and the
 // column extent of each non-empty row (autotune.cu).

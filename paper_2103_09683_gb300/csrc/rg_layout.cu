@@ -735,9 +735,7 @@ void free_row_groups(RowGroups& R) {
 // per warp: contiguous runs of equal cost left the busiest warp 25-45 % above
 // the mean, this 3-8 %).  The pieces of one group stay together; a warp takes
 // its packets in their order in memory.
-cudaError_t rg_deal(RowGroups& R, int which, uint32_t nw) {
-    RgDeal& D = R.deal[which];
-    if (D.begin && D.nw == nw) return cudaSuccess;
+cudaError_t rg_deal(const RowGroups& R, uint32_t nw, RgDeal& D) {
     const uint32_t np = (uint32_t)R.host_pk.size();
     std::vector<uint32_t> b((size_t)R.grid * nw + 1, 0);
     std::vector<uint4> pk;
@@ -786,13 +784,9 @@ cudaError_t rg_deal(RowGroups& R, int which, uint32_t nw) {
         cudaFree(dev_p);
         return e;
     }
-    R.bytes -= D.begin ? ((size_t)R.grid * D.nw + 1) * 4 + (size_t)np * 16 : 0;
-    cudaFree(D.begin);
-    cudaFree(D.pk);
     D.begin = dev_b;
     D.pk = dev_p;
     D.nw = nw;
-    R.bytes += b.size() * 4 + (size_t)np * 16;
     return cudaSuccess;
 }
 
@@ -1063,15 +1057,43 @@ uint32_t rg_warps(const dose_matrix* A, int which, uint32_t* depth, size_t* smem
                : rg_forward_warps(A, which, depth, smem);
 }
 
-// Warps of each call and the deals of packets to them (re-run when the tuning changes).
-cudaError_t rg_schedule(dose_matrix* A) {
+// Warps of each call under the knobs t and the deals of packets to them.  The knobs
+// and deals in effect are replaced when all the new ones are there: after a failure
+// every call runs as before.
+cudaError_t rg_schedule(dose_matrix* A, const AdjTuning& t) {
+    const AdjTuning old = A->adj_tuning;
+    A->adj_tuning = t;
+    RgDeal fresh[RG_DEALS];
     uint32_t depth = 0;
     size_t smem = 0;
     cudaError_t e = cudaSuccess;
+    auto layout = [&](int which) -> RowGroups& { return which == RG_DEAL_FUSED && A->rgf.built ? A->rgf : A->rg; };
     for (int which = 0; which < RG_DEALS && e == cudaSuccess; ++which) {
-        const uint32_t nw = rg_warps(A, which, &depth, &smem);
-        if (nw) e = rg_deal(which == RG_DEAL_FUSED && A->rgf.built ? A->rgf : A->rg, which, nw);
+        const RowGroups& R = layout(which);
+        const uint32_t nw = R.built ? rg_warps(A, which, &depth, &smem) : 0;
+        try {
+            if (nw && nw != R.deal[which].nw) e = rg_deal(R, nw, fresh[which]);
+        } catch (const std::exception&) {  // host memory for the lists
+            e = cudaErrorMemoryAllocation;
+        }
     }
+    for (int which = 0; which < RG_DEALS; ++which) {
+        RowGroups& R = layout(which);
+        RgDeal& D = R.deal[which];
+        const RgDeal n = fresh[which];
+        if (!n.begin) continue;
+        if (e == cudaSuccess) {
+            auto bytes = [&](const RgDeal& d) { return d.begin ? ((size_t)R.grid * d.nw + 1) * 4 + R.host_pk.size() * 16 : 0; };
+            R.bytes = R.bytes - bytes(D) + bytes(n);
+            cudaFree(D.begin);
+            cudaFree(D.pk);
+            D = n;
+        } else {
+            cudaFree(n.begin);
+            cudaFree(n.pk);
+        }
+    }
+    if (e != cudaSuccess) A->adj_tuning = old;
     return e;
 }
 

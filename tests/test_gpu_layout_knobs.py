@@ -126,3 +126,22 @@ def test_no_memory_for_the_fused_copy_keeps_the_layout(monkeypatch):
     adj_check(g.cpu().numpy(), oracle.spmv_t(n, 1600, rp, col, enc.decoded, r_own),
               oracle.abs_spmv_t(n, 1600, rp, col, enc.decoded, r_own))
     A.device_status()
+
+
+@pytest.mark.parametrize("long_rows", [True, False])
+def test_knobs_that_do_not_fit_change_nothing(monkeypatch, long_rows):
+    """dose_set_tuning without memory for the new deals or schedules (the limit lets
+    some of them through): the handle reports and computes what it did before."""
+    csr = _long_rows() if long_rows else dosegen.generate(dosegen.TINY)
+    A, _ = make(csr, "u16")
+    info, first = A.info(), _outputs(A, csr)
+    for limit in (15, 1000, 3000):
+        monkeypatch.setenv("DOSE_TEST_ALLOC_LIMIT", str(limit))
+        with pytest.raises(dose.DoseError) as ei:
+            A.set_tuning(rg_warps=2, adj_tile_nnz=512, tile_nnz=2048)
+        monkeypatch.delenv("DOSE_TEST_ALLOC_LIMIT")
+        assert ei.value.status == 2
+        assert A.info() == info
+        for a, b in zip(first, _outputs(A, csr)):
+            assert torch.equal(a, b)
+    A.device_status()
