@@ -82,6 +82,11 @@ __device__ __forceinline__ void bulk_store_wait() {
 // waits for the kernels before it: x and the other vectors are read, and
 // results written, only after rg_wait_previous().  Back-to-back calls then hide
 // the launch and the first loads' latency (3 to 5 us a call).
+// The caller's vectors may thus be written while a kernel that reads them is
+// already running: they are read by ordinary loads after the wait (which the
+// compiler does not move across it), never through the read-only path, whose data
+// must not change while the kernel runs.  x, which a projected-gradient step
+// rewrites in place, is read past L1.
 __device__ __forceinline__ void rg_let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void rg_wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

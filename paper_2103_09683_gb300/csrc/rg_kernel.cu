@@ -90,8 +90,8 @@ struct RgVecs {
             if (k && !__any_sync(0xffffffffu, rown[1] != 0xFFFFFFFFu)) break;  // most packets hold at most 32 rows
             v0n[k] = v1n[k] = 0.f;
             if (rown[k] != 0xFFFFFFFFu) {
-                v0n[k] = __ldg(p.v0 + rown[k]);
-                if (QUAD) v1n[k] = __ldg(p.v1 + rown[k]);
+                v0n[k] = p.v0[rown[k]];
+                if (QUAD) v1n[k] = p.v1[rown[k]];
             }
         }
     }
@@ -128,8 +128,8 @@ __device__ __forceinline__ void rg_empty_rows(const RgParams& p, uint32_t z, uin
     constexpr uint32_t U = 4;
     const uint32_t nq = (p.A.nrows + 3) / 4, full_q = p.A.nrows / 4;
     const uint32_t q0 = (uint32_t)((uint64_t)nq * blockIdx.x / gridDim.x), q1 = (uint32_t)((uint64_t)nq * (blockIdx.x + 1) / gridDim.x);
-    const float4* __restrict__ p4 = reinterpret_cast<const float4*>(p.v0);
-    const float4* __restrict__ w4 = reinterpret_cast<const float4*>(p.v1);
+    const float4* p4 = reinterpret_cast<const float4*>(p.v0);
+    const float4* w4 = reinterpret_cast<const float4*>(p.v1);
     for (uint32_t i0 = q0 + 32 * U * z + lane; i0 < q1; i0 += 32 * U * kRgRowWarps) {
         uint32_t m[U];
         float4 a[U], b[U];
@@ -140,14 +140,14 @@ __device__ __forceinline__ void rg_empty_rows(const RgParams& p, uint32_t z, uin
             if (i < q1 && r + 4 > p.A.nrows) m[k] |= (0xFu << (p.A.nrows - r)) & 0xFu;  // rows past the end
             a[k] = b[k] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (i < q1 && i < full_q) {
-                a[k] = __ldg(p4 + i);
-                b[k] = __ldg(w4 + i);
+                a[k] = p4[i];
+                b[k] = w4[i];
             } else if (i < q1) {
                 float t[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
                 for (uint32_t u = 0; u < 4; ++u)
                     if (r + u < p.A.nrows) {
-                        t[u] = __ldg(p.v0 + r + u);
-                        t[4 + u] = __ldg(p.v1 + r + u);
+                        t[u] = p.v0[r + u];
+                        t[4 + u] = p.v1[r + u];
                     }
                 a[k] = make_float4(t[0], t[1], t[2], t[3]);
                 b[k] = make_float4(t[4], t[5], t[6], t[7]);
@@ -273,7 +273,7 @@ __global__ void __launch_bounds__((kRgMaxWarps + kRgRowWarps) * 32, 1) rg_kernel
     if (!(p.chain & RG_CHAIN_PREV)) rg_wait_previous();
     if (p.chain & RG_CHAIN_NEXT) rg_let_next_start();
     if (QUAD) {
-        C.each(t, T, [&](uint32_t j, uint32_t c) { xs[j] = __ldg(p.x + c); });
+        C.each(t, T, [&](uint32_t j, uint32_t c) { xs[j] = __ldcg(p.x + c); });
         if (t == 0) xs[nc] = 0.f;
     }
     if (warp < NW) V.values(p);

@@ -66,7 +66,7 @@ __global__ void __launch_bounds__((kMvWorkers + 1) * 32, 1) rg_spmv_kernel(const
     }
     const uint32_t nc = C.nc;
     rg_wait_previous();
-    C.each(t, T, [&](uint32_t j, uint32_t c) { xs[j] = __ldg(static_cast<const float*>(p.x) + c); });
+    C.each(t, T, [&](uint32_t j, uint32_t c) { xs[j] = __ldcg(static_cast<const float*>(p.x) + c); });
     if (t == 0) xs[nc] = 0.f;
     __syncthreads();
     float* __restrict__ d = static_cast<float*>(p.d);
@@ -230,7 +230,7 @@ __global__ void __launch_bounds__((kMv64Workers + 1) * 32, 1) rg_spmv64_kernel(c
     }
     const uint32_t nc = C.nc;
     rg_wait_previous();
-    C.each(t, T, [&](uint32_t j, uint32_t c) { xs[j] = prepare_x<MODE>(__ldg(static_cast<const double*>(p.x) + c)); });
+    C.each(t, T, [&](uint32_t j, uint32_t c) { xs[j] = prepare_x<MODE>(__ldcg(static_cast<const double*>(p.x) + c)); });
     if (t == 0) xs[nc] = make_uint2(0u, 0u);
     __syncthreads();
     if (warp >= NW) {
@@ -356,7 +356,7 @@ __global__ void __launch_bounds__((kMmWorkers[0] + 1) * 32, 1) rg_spmm_kernel(co
         for (uint32_t j = threadIdx.x; j < (nc + 1) * 4 * NQ; j += nct) {
             const uint32_t c = j / (4 * NQ), v = j % (4 * NQ);
             xs[mm_x<NQ>(c, v >> 2) + (v & 3u)] =
-                c < nc && v < p.nvec ? __ldg(it.X + (size_t)__ldg(C.dict + c) * p.nvec + v) : 0.f;
+                c < nc && v < p.nvec ? __ldcg(it.X + (size_t)__ldg(C.dict + c) * p.nvec + v) : 0.f;
         }
         dev::named_barrier(1, nct);
         const bool vec4 = (p.nvec & 3u) == 0 && (reinterpret_cast<uintptr_t>(it.D) & 15u) == 0;
