@@ -554,6 +554,12 @@ static dose_status make_schedule(const dose_matrix* A, uint32_t grid, const Tuni
     D.n_coop_rows = S.n_coop_rows;
     std::memcpy(D.lanes_hist, S.lanes_hist, sizeof(D.lanes_hist));
     D.tuning = t;
+    // a copy from pageable memory may return before it has reached the device, and a
+    // caller's stream need not wait for the default one
+    if ((e = cudaStreamSynchronize(nullptr)) != cudaSuccess) {
+        free_dev_schedule(D);
+        return cuda_fail(e, "uploading the schedule");
+    }
     return DOSE_OK;
 }
 

@@ -1077,6 +1077,7 @@ cudaError_t rg_schedule(dose_matrix* A, const AdjTuning& t) {
             e = cudaErrorMemoryAllocation;
         }
     }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);  // the copies have reached the device
     for (int which = 0; which < RG_DEALS; ++which) {
         RowGroups& R = layout(which);
         RgDeal& D = R.deal[which];
