@@ -417,7 +417,7 @@ __global__ void __launch_bounds__(256) adjoint_finalize(const float* __restrict_
 template <int FMT, int MODE>
 cudaError_t launch_adj_t(const dose_matrix* A, const AdjParams& p, size_t smem, cudaStream_t s) {
     auto k = adjoint_kernel<FMT, MODE>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_max_smem(k);
     if (e != cudaSuccess) return e;
     const uint32_t warps = 1 + (MODE == ADJ_MODE_QUADRATIC ? p.fwarps : 0) + p.swarps;
     k<<<A->adj.grid, 32 * warps, smem, s>>>(p);

@@ -485,7 +485,7 @@ cudaError_t launch_staged(const dose_matrix* const* A, const float* const* X, fl
         p.l2pf = std::max(p.l2pf, M->adj_tuning.l2_prefetch);
     }
     auto k = spmm_staged_kernel<NQ>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_max_smem(k);
     if (e != cudaSuccess) return e;
     k<<<A[0]->adj.grid, 32 * (kSpmmConsumerWarps + 1), smem, s>>>(p);
     return cudaGetLastError();

@@ -370,6 +370,13 @@ Tuning adj_schedule_tuning(const Tuning& fwd, const AdjTuning& a);
 uint64_t matrix_fingerprint(const dose_matrix* A);
 
 constexpr uint32_t kMaxSmemPerBlock = 227 * 1024;
+// Lets a kernel without static shared memory use all of a block's.  Always the same
+// limit, never the size of the call at hand: another thread's call could lower that
+// between this one's limit and its launch.
+template <class K>
+cudaError_t allow_max_smem(K k) {
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmemPerBlock);
+}
 
 // Stored bytes per value of a format.
 __host__ __device__ constexpr uint32_t value_bytes(int fmt) {

@@ -175,7 +175,7 @@ extern "C" dose_status dose_adjoint_noalloc(uint32_t nrows, uint32_t ncols, uint
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const size_t smem = (size_t)W * ncols * 4;
     if (smem > 48 * 1024) {
-        e = cudaFuncSetAttribute(noalloc_adjoint_partials, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = allow_max_smem(noalloc_adjoint_partials);
         if (e != cudaSuccess) return cuda_fail(e, "dose_adjoint_noalloc: shared memory attribute");
     }
     noalloc_adjoint_partials<<<P, 32 * W, smem, s>>>(nrows, ncols, nnz, row_ptr, col_idx, (int)fmt, values,

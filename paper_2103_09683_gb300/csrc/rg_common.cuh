@@ -31,7 +31,7 @@ constexpr uint32_t kRgZeroBytes = 4096;    // zeros that the bulk stores of rows
 template <class K, class P>
 cudaError_t rg_launch(K k, const P& p, dim3 grid, uint32_t threads, size_t smem, cudaStream_t s, bool early = true) {
     if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = allow_max_smem(k);
         if (e != cudaSuccess) return e;
     }
     cudaLaunchConfig_t cfg = {};

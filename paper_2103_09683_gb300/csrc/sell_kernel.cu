@@ -161,7 +161,7 @@ cudaError_t launch_t(const dose_matrix* A, const SellParams& p, cudaStream_t s) 
     const bool comp = (A->flags & DOSE_CREATE_COMPENSATED) != 0;
     auto k = xsmem ? (comp ? sell_spmv_kernel<FMT, IW, true, true> : sell_spmv_kernel<FMT, IW, true, false>)
                    : (comp ? sell_spmv_kernel<FMT, IW, false, true> : sell_spmv_kernel<FMT, IW, false, false>);
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_max_smem(k);
     if (e != cudaSuccess) return e;
     const uint32_t grid = std::max(1u, std::min<uint32_t>((uint32_t)A->sm_count * kSellCtasPerSm,
                                                           (A->sell.nchunks + kSellWarps - 1) / kSellWarps));

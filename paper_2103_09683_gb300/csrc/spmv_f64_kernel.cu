@@ -242,7 +242,7 @@ __global__ void __launch_bounds__(544, 1) spmv_f64_kernel(const Spmv64Params p) 
 template <int FMT, int MODE, bool XSMEM, uint32_t IW>
 cudaError_t launch_t(const dose_matrix* A, const Spmv64Params& p, size_t smem, cudaStream_t s) {
     auto k = spmv_f64_kernel<FMT, MODE, XSMEM, IW>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_max_smem(k);
     if (e != cudaSuccess) return e;
     k<<<(A->fwd64_own ? A->fwd64 : A->fwd).grid, 32 * (p.cwarps + 1), smem, s>>>(p);
     return cudaGetLastError();

@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(544, 1) spmv_kernel(const SpmvParams p) {
 template <int FMT, bool COMP, bool XSMEM, uint32_t IW>
 cudaError_t launch_t(const dose_matrix* A, const SpmvParams& p, size_t smem, cudaStream_t s) {
     auto k = spmv_kernel<FMT, COMP, XSMEM, IW>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_max_smem(k);
     if (e != cudaSuccess) return e;
     k<<<A->fwd.grid, 32 * (p.cwarps + 1), smem, s>>>(p);
     return cudaGetLastError();
