@@ -485,6 +485,7 @@ Schedule kept_schedule(const Csr& A, const std::vector<uint32_t>& rows, const st
 // into loc.
 struct BankOrder {
     std::vector<uint32_t> cap, has, at;
+    uint16_t step_of[kMaxRowEntries];
     // blocks: also arrange each step for the batched SpMM's gathers
     void operator()(const uint32_t* loc, uint32_t n, uint32_t* perm, bool blocks) {
         const uint32_t steps = (n + 31) / 32;
@@ -515,34 +516,33 @@ struct BankOrder {
                 if (best < 0)
                     for (uint32_t s = 0; s < steps; ++s)
                         if (cap[s] && (best < 0 || cap[s] > cap[best])) best = (int)s;
-                perm[32 * best + at[best]++] = item[k];
+                step_of[item[k]] = (uint16_t)best;
                 --cap[best];
                 has[best] |= 1u << b;
             }
         }
+        for (uint32_t i = 0; i < n; ++i) perm[32 * step_of[i] + at[step_of[i]]++] = i;  // ascending inside a step
+        if (!blocks) return;
         // inside a step: eight consecutive positions with columns that differ mod 8
         // where that is possible (the batched SpMM's 16-byte X gathers: without it 37 %
-        // of its shared-memory wavefronts were bank conflicts)
+        // of its shared-memory wavefronts were bank conflicts): the first column left of
+        // each residue, then (no other residues left) the first columns left
         for (uint32_t s = 0; s < steps; ++s) {
             uint32_t* p = perm + 32 * s;
-            std::sort(p, p + at[s]);
-            if (!blocks) continue;
-            uint32_t tmp[32], used = 0, k = 0;
-            while (k < at[s]) {
-                uint32_t seen = 0, in_block = 0;
-                for (uint32_t i = 0; i < at[s] && in_block < 8; ++i)
-                    if (!((used >> i) & 1u) && !((seen >> (loc[p[i]] & 7u)) & 1u)) {
-                        seen |= 1u << (loc[p[i]] & 7u);
-                        used |= 1u << i;
-                        tmp[k++] = p[i];
-                        ++in_block;
-                    }
-                for (uint32_t i = 0; i < at[s] && in_block < 8; ++i)  // (no other residues left)
-                    if (!((used >> i) & 1u)) {
-                        used |= 1u << i;
-                        tmp[k++] = p[i];
-                        ++in_block;
-                    }
+            uint32_t of[8] = {0}, tmp[32], left = 0, k = 0;  // positions left, by residue and in all
+            for (uint32_t i = 0; i < at[s]; ++i) of[loc[p[i]] & 7u] |= 1u << i;
+            for (uint32_t q = 0; q < 8; ++q) left |= of[q];
+            while (left) {
+                uint32_t pick = 0, in_block = 0;
+                for (uint32_t q = 0; q < 8; ++q) pick |= of[q] & (0u - of[q]);
+                while (in_block < 8 && left) {
+                    const uint32_t from = pick ? pick : left, bit = from & (0u - from), i = (uint32_t)__builtin_ctz(bit);
+                    of[loc[p[i]] & 7u] &= ~bit;
+                    left &= ~bit;
+                    pick &= ~bit;
+                    tmp[k++] = p[i];
+                    ++in_block;
+                }
             }
             std::copy(tmp, tmp + at[s], p);
         }
@@ -579,7 +579,8 @@ void write_cta(const Csr& A, uint32_t hr, uint32_t iw, uint32_t cap, uint32_t ma
         }
     std::sort(out.dict.begin(), out.dict.end());
     for (uint32_t i = 0; i < out.dict.size(); ++i) pos[out.dict[i]] = i;  // global column -> local
-    std::vector<uint32_t> loc, perm, at(out.dict.size(), 0);
+    std::vector<uint32_t> loc, perm;
+    std::vector<size_t> where(out.dict.size());  // where a column's values lie in out.data
     BankOrder order;
     struct Piece {
         const Grp* g;
@@ -588,7 +589,22 @@ void write_cta(const Csr& A, uint32_t hr, uint32_t iw, uint32_t cap, uint32_t ma
     std::vector<Piece> open;
     std::vector<std::vector<uint32_t>> open_loc;  // each piece's local columns in stored order
     uint32_t open_u = 0;
-    auto flush = [&](uint32_t flags) -> size_t {
+    auto put_values = [&](const Grp& g) {
+        for (uint32_t s = 0; s < g.cnt; ++s) {
+            const uint32_t r = rows[g.first + s];
+            for (uint32_t k = A.rp[r]; k < A.rp[r + 1]; ++k) {
+                unsigned char* o = out.data.data() + where[pos[A.col[k]]] + (size_t)s * A.es;
+                if (A.es == 2)
+                    std::memcpy(o, A.vals + 2 * (size_t)k, 2);
+                else if (A.es == 1)
+                    *o = A.vals[k];
+                else
+                    std::memcpy(o, A.vals + 4 * (size_t)k, 4);
+            }
+        }
+    };
+    // values: write the groups' values (else, for a piece, only note where they go)
+    auto flush = [&](uint32_t flags, bool values) -> size_t {
         const uint32_t ng = (uint32_t)open.size();
         const RgPacket L = rg_packet(ng, open_u, hr, iw, A.es, fp8);
         const size_t base = out.data.size();
@@ -616,24 +632,9 @@ void write_cta(const Csr& A, uint32_t hr, uint32_t iw, uint32_t cap, uint32_t ma
                     reinterpret_cast<uint16_t*>(p + L.cols)[u + k] = (uint16_t)lc[k];
                 else
                     reinterpret_cast<uint32_t*>(p + L.cols)[u + k] = lc[k];
-                at[lc[k]] = k + 1;
+                where[lc[k]] = base + L.vals + ((size_t)u + k) * hr * A.es;
             }
-            unsigned char* vo = p + L.vals + (size_t)u * hr * A.es;
-            for (uint32_t s = 0; s < g.cnt; ++s) {
-                const uint32_t r = rows[g.first + s];
-                for (uint32_t k = A.rp[r]; k < A.rp[r + 1]; ++k) {
-                    const uint32_t q = at[pos[A.col[k]]];  // 0: in another piece
-                    if (!q) continue;
-                    const size_t o = (size_t)(q - 1) * hr + s;
-                    if (A.es == 2)
-                        std::memcpy(vo + 2 * o, A.vals + 2 * (size_t)k, 2);
-                    else if (A.es == 1)
-                        vo[o] = A.vals[k];
-                    else
-                        std::memcpy(vo + 4 * o, A.vals + 4 * (size_t)k, 4);
-                }
-            }
-            for (uint32_t k = 0; k < n; ++k) at[lc[k]] = 0;
+            if (values) put_values(g);
             u += n;
         }
         const uint32_t* ro = reinterpret_cast<const uint32_t*>(p + L.rows);
@@ -662,7 +663,7 @@ void write_cta(const Csr& A, uint32_t hr, uint32_t iw, uint32_t cap, uint32_t ma
         }
         const uint32_t np = (g.nu + max_u - 1) / max_u;
         if (!open.empty() && (np > 1 || open_u + g.nu > cap || open.size() >= max_g || (keep && (*keep)[gi] != (*keep)[gi - 1]))) {
-            flush(RG_FORWARD | RG_SCATTER);
+            flush(RG_FORWARD | RG_SCATTER, true);
             if (keep) out.tag.resize(out.pk.size(), (*keep)[gi - 1]);
         }
         std::vector<size_t> piece_pk;
@@ -681,8 +682,12 @@ void write_cta(const Csr& A, uint32_t hr, uint32_t iw, uint32_t cap, uint32_t ma
             open_loc.push_back(std::move(lc));
             open_u += hi - lo;
             if (np > 1)
-                piece_pk.push_back(flush(RG_FORWARD | (i ? RG_CARRY_IN : 0u) | (i + 1 < np ? RG_CARRY_OUT : RG_SCATTER)));
+                piece_pk.push_back(flush(RG_FORWARD | (i ? RG_CARRY_IN : 0u) | (i + 1 < np ? RG_CARRY_OUT : RG_SCATTER), false));
         }
+        // the values of a group of several pieces, once over its rows (piece by piece, each
+        // over all entries, the layout of the beam shaped like the paper's liver beam 1
+        // took 3.5 times as long to write)
+        if (np > 1) put_values(g);
         // a group of several pieces: its residuals are known after the last one, so
         // the earlier pieces come once more for the scatter
         for (uint32_t i = 0; again && i + 1 < np; ++i) {
@@ -692,7 +697,7 @@ void write_cta(const Csr& A, uint32_t hr, uint32_t iw, uint32_t cap, uint32_t ma
         }
         if (keep) out.tag.resize(out.pk.size(), (*keep)[gi]);
     }
-    if (!open.empty()) flush(RG_FORWARD | RG_SCATTER);
+    if (!open.empty()) flush(RG_FORWARD | RG_SCATTER, true);
     if (keep && !keep->empty()) out.tag.resize(out.pk.size(), keep->back());
 }
 
