@@ -219,7 +219,9 @@ typedef struct {
     uint32_t rg_window;         /* most columns any CTA sees on the row-group layout */
     uint32_t rg_warps_fused;    /* worker warps of the row-group fused pass (0 if it does not fit) */
     uint32_t rg_index_bytes;    /* bytes per union column index (2 when ncols <= 65536, else 4) */
-    uint32_t rg_pad;
+    uint16_t rg_rows;           /* rows per group: 8 or 4 */
+    uint16_t rg_order;          /* row order: 0 as stored, 1 along the beam (plane by plane in lateral tiles),
+                                   2 cubes of 2 x 2 x 2 voxels, 3 by first and last column */
     uint64_t fingerprint;       /* FNV-1a of the structure (dose_fingerprint_host): the autotune cache key */
     uint32_t spmv_layout;       /* layout dose_spmv runs on: 1 = CSR, 2 = row groups, 3 = SELL */
     uint32_t pad2;

@@ -86,7 +86,8 @@ class _Info(ctypes.Structure):
                 ("adj_layout_fused", ctypes.c_uint32), ("adj_layout_adjoint", ctypes.c_uint32),
                 ("rg_groups", ctypes.c_uint64), ("rg_union_entries", ctypes.c_uint64),
                 ("rg_window", ctypes.c_uint32), ("rg_warps_fused", ctypes.c_uint32),
-                ("rg_index_bytes", ctypes.c_uint32), ("rg_pad", ctypes.c_uint32), ("fingerprint", ctypes.c_uint64),
+                ("rg_index_bytes", ctypes.c_uint32), ("rg_rows", ctypes.c_uint16),
+                ("rg_order", ctypes.c_uint16), ("fingerprint", ctypes.c_uint64),
                 ("spmv_layout", ctypes.c_uint32), ("pad2", ctypes.c_uint32), ("rg_spmv_bytes", ctypes.c_uint64)]
 
 

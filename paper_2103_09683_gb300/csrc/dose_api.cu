@@ -1257,6 +1257,8 @@ dose_status dose_matrix_info(const dose_matrix* A, dose_info* out) {
         out->rg_union_entries = A->rg.n_union * A->rg.hr / 4;
         out->rg_window = A->rg.wmax;
         out->rg_index_bytes = A->rg.iw;
+        out->rg_rows = (uint16_t)A->rg.hr;
+        out->rg_order = (uint16_t)A->rg.order;
         out->tuning.rg_tile_union = A->adj_tuning.rg_tile_u ? A->adj_tuning.rg_tile_u : A->rg.tile_u;
         out->rg_warps_fused = rg_gradient_warps(A, A->adj_tuning, true, nullptr, nullptr);
         if (rg_active(A, true)) {
