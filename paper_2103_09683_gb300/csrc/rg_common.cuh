@@ -103,13 +103,28 @@ struct RgDict {
 #pragma unroll
         for (uint32_t k = 0; k < 2; ++k) c[k] = t + k * nt < nc ? __ldg(dict + t + k * nt) : 0u;
     }
-    // put(j, column) for this thread's columns j = t, t + nt, ...
-    template <class F>
-    __device__ __forceinline__ void each(uint32_t t, uint32_t nt, F put) const {
+    // put(j, get(column)) for this thread's columns j = t, t + nt, ...; four columns,
+    // then four values in flight past the first two (a list of 25,000 columns is
+    // some thirty rounds of both)
+    template <class G, class P>
+    __device__ __forceinline__ void each(uint32_t t, uint32_t nt, G get, P put) const {
+        decltype(get(0u)) v[4];
 #pragma unroll
         for (uint32_t k = 0; k < 2; ++k)
-            if (t + k * nt < nc) put(t + k * nt, c[k]);
-        for (uint32_t j = t + 2 * nt; j < nc; j += nt) put(j, __ldg(dict + j));
+            if (t + k * nt < nc) v[k] = get(c[k]);
+#pragma unroll
+        for (uint32_t k = 0; k < 2; ++k)
+            if (t + k * nt < nc) put(t + k * nt, v[k]);
+        for (uint32_t j = t + 2 * nt; j < nc; j += 4 * nt) {
+            uint32_t q[4];
+#pragma unroll
+            for (uint32_t k = 0; k < 4; ++k) q[k] = __ldg(dict + min(j + k * nt, nc - 1));
+#pragma unroll
+            for (uint32_t k = 0; k < 4; ++k) v[k] = get(q[k]);
+#pragma unroll
+            for (uint32_t k = 0; k < 4; ++k)
+                if (j + k * nt < nc) put(j + k * nt, v[k]);
+        }
     }
 };
 

@@ -273,7 +273,7 @@ __global__ void __launch_bounds__((kRgMaxWarps + kRgRowWarps) * 32, 1) rg_kernel
     if (!(p.chain & RG_CHAIN_PREV)) rg_wait_previous();
     if (p.chain & RG_CHAIN_NEXT) rg_let_next_start();
     if (QUAD) {
-        C.each(t, T, [&](uint32_t j, uint32_t c) { xs[j] = __ldcg(p.x + c); });
+        C.each(t, T, [&](uint32_t c) { return __ldcg(p.x + c); }, [&](uint32_t j, float v) { xs[j] = v; });
         if (t == 0) xs[nc] = 0.f;
     }
     if (warp < NW) V.values(p);

@@ -66,7 +66,8 @@ __global__ void __launch_bounds__((kMvWorkers + 1) * 32, 1) rg_spmv_kernel(const
     }
     const uint32_t nc = C.nc;
     rg_wait_previous();
-    C.each(t, T, [&](uint32_t j, uint32_t c) { xs[j] = __ldcg(static_cast<const float*>(p.x) + c); });
+    C.each(t, T, [&](uint32_t c) { return __ldcg(static_cast<const float*>(p.x) + c); },
+           [&](uint32_t j, float v) { xs[j] = v; });
     if (t == 0) xs[nc] = 0.f;
     __syncthreads();
     float* __restrict__ d = static_cast<float*>(p.d);
@@ -230,7 +231,8 @@ __global__ void __launch_bounds__((kMv64Workers + 1) * 32, 1) rg_spmv64_kernel(c
     }
     const uint32_t nc = C.nc;
     rg_wait_previous();
-    C.each(t, T, [&](uint32_t j, uint32_t c) { xs[j] = prepare_x<MODE>(__ldcg(static_cast<const double*>(p.x) + c)); });
+    C.each(t, T, [&](uint32_t c) { return __ldcg(static_cast<const double*>(p.x) + c); },
+           [&](uint32_t j, double v) { xs[j] = prepare_x<MODE>(v); });
     if (t == 0) xs[nc] = make_uint2(0u, 0u);
     __syncthreads();
     if (warp >= NW) {
