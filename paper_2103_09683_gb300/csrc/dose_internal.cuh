@@ -171,10 +171,11 @@ struct RowGroups {
     uint32_t grid = 0;              // CTAs the groups are cut for
     uint32_t hr = 8;                // rows per group (values stored per union column)
     uint32_t iw = 4;                // bytes per stored column index (2 when ncols <= 65536)
-    uint32_t order = 0;             // row order taken (rg_layout.cu)
+    uint32_t order = 0;             // row order taken (rg_layout.cu), on a grid of these strides
+    uint32_t line = 0, plane = 0;
     bool forward_only = false;      // rows too long for the gradient passes: dose_spmv, dose_spmv_f64 and the
                                     //   batched SpMM only
-    bool keep = false;              // the stored-row order of the fused pass (rg_layout.cu), cut for
+    bool keep = false;              // the stored-row deal of the fused pass (rg_layout.cu), cut for
     uint32_t keep_nw = 0;           //   this many warps per CTA
     std::vector<uint32_t> keep_tag; //   each packet's warp
     uint64_t n_groups = 0, n_union = 0;
@@ -388,14 +389,21 @@ constexpr uint32_t kRgRowWarps = 3;        // more warps of the fused pass, for 
 constexpr uint32_t kRgDefaultUnion = 320;  // union columns of a packet (6 KB with eight 16-bit values each)
 constexpr uint32_t kRgMaxRows = 64;        // rows of a packet
 constexpr uint32_t kRgZeroRun = 1024;      // rows of a run without entries
-// The fused pass keeps the stored-row order up to this many rows with entries (rg_layout.cu):
-// beyond, another order moves f by at most 4e-10 of itself (measured on beams of 0.5 to 7e5
-// rows).  A plan of several beams has doses near the prescription and so an f of small
-// differences (moved by up to 3e-9 on 1.5e5 rows, 1.4e-9 on 4e5 to 8e5): it keeps the order longer.
-// Large plans do not, as it costs them more than half the step (nine scenarios of a 160 x
-// 160 x 100 plan, 8e5 rows: 2.30 ms in the kept order, 0.94 in the new one, 1.90 with the
-// stage-ring kernels).
+// Rows with entries up to which the fused pass keeps the stored-row order of each
+// row's sum (rg_layout.cu), on single beams and on plans of several.  Another order
+// moves f by at most 5e-10 of itself on beams of 5e4 to 7e5 rows, and by up to 3e-9 on
+// plans of 1.5e5 (their doses are near the prescription, so that f is made of small
+// differences); 100 projected-gradient steps on a beam carry it on to 2e-9 to 5e-9 (1e-8
+// on 1e4 rows).  The lines are drawn by cost as well: on beams the kept order (at its best
+// deal) costs a quarter of the pass from 2e5 rows on (objective on 1.85e5 rows, u16: 31
+// us, 23 in the other order), so the smaller move decides from there; plans of 4e5
+// rows and more move f by up to 1.4e-9 but pay more than half the step for the kept
+// order (nine scenarios of a 160 x 160 x 100 plan: 2.30 ms, 0.94 in the other order).
 constexpr uint32_t kRgKeepRows = 200000, kRgKeepPlanRows = 400000;
+// ... and up to which it keeps the deal of the groups to CTAs and warps too: by 1e5 rows
+// the kept deal's lead over the kernels it replaced is gone (plan of 1e5 rows, F32: 37.1
+// us against 37.0; beams of 1.0e5 to 1.3e5 rows are still 7 to 28 % ahead).
+constexpr uint32_t kRgKeepDealRows = 100000;
 constexpr uint32_t kMaxAdjWarps = 20;      // producer + forward + scatter warps of the adjoint kernels
 constexpr uint32_t kSellDefaultSigma = 1u << 20;  // rows per sorting window of the SELL copy
 constexpr uint32_t kAdjMinScatterWarps = 8;

@@ -387,10 +387,20 @@ struct Grp {
 // do not (up to 3e-9 on small plans, 1e-8 after 100 steps).  So the fused pass of
 // small matrices (kRgKeepRows, kRgKeepPlanRows) keeps one fixed order, whatever order
 // the other passes' groups take: groups of up to four consecutive non-empty rows,
-// cut into stages of consecutive groups, stages dealt to CTAs by column windows
-// and the groups of a stage dealt round-robin to the warps, a step further at
-// each stage.  Groups, stages and deals below define that order; nothing else
-// depends on them.
+// each group's columns in one order.  These alone set the doses, and with them f (its
+// terms are added in double-float and FP64).
+// The gradient's rounding, which a projected-gradient loop feeds back, follows the
+// deal of the groups as well.  Small matrices keep that too: stages of consecutive
+// groups, dealt to CTAs by column windows, and the groups of a stage round-robin to
+// the warps, a step further at each stage.  From kRgKeepDealRows rows on, where its
+// uneven shares and small packets (a shared-memory slot for each of fifteen warps, so
+// unions cut in pieces that are read twice) made the fused pass slower than the
+// stage-ring kernels, the kept groups are dealt like the other layout's.
+// Objective on F32 beams and three-beam plans, stage rings / kept deal / this: 1.7e5 rows
+// F32 38.6 / 39.2 / 32.6 us; plans of 1.5e5 rows u16 39.1 / 39.1 / 36.9, F32 49.4 / 51.3 /
+// 41.6; of 2.2e5 rows u16 59.6 / 65.8 / 57.9, F32 79.6 / 93.0 / 67.7.  Same d, f to 6e-16.
+// FP8, whose unions fit the packets, is faster on the kept deal (1.7e5 rows: 33.0 /
+// 28.9 / 30.9) and stays on it.
 
 // Groups of up to four consecutive non-empty rows within 255 rows whose union
 // stays within 320 columns and grows by at most half.
@@ -562,10 +572,10 @@ struct CtaOut {
 
 
 // cap: union columns a packet of several groups may hold; max_u: ... a packet of
-// one.  keep (each group's warp): packets hold groups of one warp, their columns
-// in the order of the stored-row layout.
+// one.  kept: a group's columns in the order of the stored-row layout; tags (each
+// group's warp): packets hold groups of one warp.
 void write_cta(const Csr& A, uint32_t hr, uint32_t iw, uint32_t cap, uint32_t max_u, const uint32_t* rows,
-               const std::vector<std::pair<const Grp*, const uint32_t*>>& groups, const std::vector<uint32_t>* keep, bool again,
+               const std::vector<std::pair<const Grp*, const uint32_t*>>& groups, bool kept, const std::vector<uint32_t>* tags, bool again,
                std::vector<uint32_t>& pos, std::vector<uint32_t>& seen, uint32_t gen, CtaOut& out) {
     const bool fp8 = A.scales != nullptr;
     // distinct columns
@@ -656,15 +666,15 @@ void write_cta(const Csr& A, uint32_t hr, uint32_t iw, uint32_t cap, uint32_t ma
         for (uint32_t k = 0; k < g.nu; ++k) loc[k] = pos[gp.second[k]];
         std::sort(loc.begin(), loc.end());
         perm.resize(g.nu);
-        if (keep) {  // banks by global column, over the whole union
+        if (kept) {  // banks by global column, over the whole union
             res.resize(g.nu);
             for (uint32_t k = 0; k < g.nu; ++k) res[k] = out.dict[loc[k]];
             order(res.data(), g.nu, perm.data(), false);
         }
         const uint32_t np = (g.nu + max_u - 1) / max_u;
-        if (!open.empty() && (np > 1 || open_u + g.nu > cap || open.size() >= max_g || (keep && (*keep)[gi] != (*keep)[gi - 1]))) {
+        if (!open.empty() && (np > 1 || open_u + g.nu > cap || open.size() >= max_g || (tags && (*tags)[gi] != (*tags)[gi - 1]))) {
             flush(RG_FORWARD | RG_SCATTER, true);
-            if (keep) out.tag.resize(out.pk.size(), (*keep)[gi - 1]);
+            if (tags) out.tag.resize(out.pk.size(), (*tags)[gi - 1]);
         }
         std::vector<size_t> piece_pk;
         for (uint32_t i = 0; i < np; ++i) {
@@ -673,7 +683,7 @@ void write_cta(const Csr& A, uint32_t hr, uint32_t iw, uint32_t cap, uint32_t ma
             const uint32_t lo = 32 * (uint32_t)((uint64_t)steps * i / np);
             const uint32_t hi = i + 1 == np ? g.nu : 32 * (uint32_t)((uint64_t)steps * (i + 1) / np);
             std::vector<uint32_t> lc(hi - lo);
-            if (!keep) {
+            if (!kept) {
                 order(loc.data() + lo, hi - lo, perm.data() + lo, true);
                 for (uint32_t k = lo; k < hi; ++k) perm[k] += lo;
             }
@@ -695,10 +705,10 @@ void write_cta(const Csr& A, uint32_t hr, uint32_t iw, uint32_t cap, uint32_t ma
             out.pk.push_back(make_uint4(q.x, (q.y & RG_SIZE_MASK) | RG_SCATTER | RG_AGAIN, q.z, q.w));
             out.cost.push_back(out.cost[piece_pk[i]]);
         }
-        if (keep) out.tag.resize(out.pk.size(), (*keep)[gi]);
+        if (tags) out.tag.resize(out.pk.size(), (*tags)[gi]);
     }
     if (!open.empty()) flush(RG_FORWARD | RG_SCATTER, true);
-    if (keep && !keep->empty()) out.tag.resize(out.pk.size(), keep->back());
+    if (tags && !tags->empty()) out.tag.resize(out.pk.size(), tags->back());
 }
 
 }  // namespace
@@ -838,6 +848,7 @@ bool build_row_groups(dose_matrix* A, RowGroups& R, bool keep, const uint32_t* r
         Order order = ORDER_MATRIX;
         bool ok = true;
         Schedule KS;
+        const bool kept_deal = keep && (rows.size() < kRgKeepDealRows || es == 1);
         if (keep) {
             R.hr = 4;
             sg.resize(1);
@@ -846,51 +857,65 @@ bool build_row_groups(dose_matrix* A, RowGroups& R, bool keep, const uint32_t* r
                 sg[0].push_back({(uint32_t)first, cnt, (uint32_t)u.size(), su[0].size()});
                 su[0].insert(su[0].end(), u.begin(), u.end());
             });
-            const AdjTuning& t = A->adj_tuning;
-            KS = kept_schedule(M, rows, sg[0], su[0], R.iw, grid, tile_u, t.rg_tile_rows, M.scales != nullptr);
-            // the warps that fitted beside this order's stages and windows; packets as
-            // large as two slots each leave room for
-            auto r128 = [](uint64_t v) { return (v + 127) / 128 * 128; };
-            const uint64_t own = r128(4ull * KS.wwidth), most = t.rg_warps ? std::min<uint32_t>(t.rg_warps, kRgMaxWarps) : kRgMaxWarps;
-            const uint64_t stage = 128 + r128(kKeepStageGroups * 16) + r128((tile_u + 16) * R.iw) + r128((tile_u + 8ull) * 4 * es) +
-                                   (M.scales ? 3 : 2) * r128((t.rg_tile_rows + 8) * 4);
-            const uint64_t rest = 3072 + r128(4ull * KS.wwidth + 4) + t.rg_stages * stage;
-            R.keep_nw = (uint32_t)(rest + own <= kMaxSmemPerBlock ? std::min<uint64_t>(most, (kMaxSmemPerBlock - rest) / own) : most);
-            const uint64_t room = (kMaxSmemPerBlock - std::min<uint64_t>(kMaxSmemPerBlock, 8192 + own)) / R.keep_nw;
-            max_u = (uint32_t)std::min<uint64_t>(kMaxRowEntries, room > own + 2560 ? (room - own - 2048) / 2 / (4 * es + R.iw) / 32 * 32 : 0);
-            max_u = std::max(max_u, 128u);
-        } else {
-        const Strides S = find_strides(M, rows, cmin, cmax);
-        choose_order(M, rows, S, cmin, cmax, R.iw, es <= 2 ? 8 : 4, order, R.hr);
-        std::vector<uint8_t> cube;
-        if (!order_rows(M, rows, order, S, cmin, cmax, &cube)) order = ORDER_MATRIX;
-        const uint32_t hr = R.hr;
-
-        // groups, formed segment by segment (four segments per CTA, about equal entries)
-        const uint32_t nseg = std::max<uint32_t>(1, std::min<uint32_t>(4 * grid, (uint32_t)(rows.size() / 256)));
-        std::vector<size_t> seg(nseg + 1, rows.size());
-        {
-            uint64_t run = 0;
-            uint32_t s = 0;
-            for (size_t i = 0; i < rows.size(); ++i) {
-                while (s < nseg && run * nseg >= (uint64_t)s * A->nnz) seg[s++] = i;
-                run += rp[rows[i] + 1] - rp[rows[i]];
+            if (kept_deal) {
+                const AdjTuning& t = A->adj_tuning;
+                KS = kept_schedule(M, rows, sg[0], su[0], R.iw, grid, tile_u, t.rg_tile_rows, M.scales != nullptr);
+                // the warps that fitted beside this order's stages and windows; packets as
+                // large as two slots each leave room for
+                auto r128 = [](uint64_t v) { return (v + 127) / 128 * 128; };
+                const uint64_t own = r128(4ull * KS.wwidth), most = t.rg_warps ? std::min<uint32_t>(t.rg_warps, kRgMaxWarps) : kRgMaxWarps;
+                const uint64_t stage = 128 + r128(kKeepStageGroups * 16) + r128((tile_u + 16) * R.iw) + r128((tile_u + 8ull) * 4 * es) +
+                                       (M.scales ? 3 : 2) * r128((t.rg_tile_rows + 8) * 4);
+                const uint64_t rest = 3072 + r128(4ull * KS.wwidth + 4) + t.rg_stages * stage;
+                R.keep_nw = (uint32_t)(rest + own <= kMaxSmemPerBlock ? std::min<uint64_t>(most, (kMaxSmemPerBlock - rest) / own) : most);
+                const uint64_t room = (kMaxSmemPerBlock - std::min<uint64_t>(kMaxSmemPerBlock, 8192 + own)) / R.keep_nw;
+                max_u = (uint32_t)std::min<uint64_t>(kMaxRowEntries, room > own + 2560 ? (room - own - 2048) / 2 / (4 * es + R.iw) / 32 * 32 : 0);
+                max_u = std::max(max_u, 128u);
+            } else {
+                // shares of the other calls' order: a CTA then sees a compact region
+                std::vector<uint32_t> sorted = rows, rank(nrows, 0);
+                Strides S;
+                S.line = A->rg.line;
+                S.plane = A->rg.plane;
+                order_rows(M, sorted, (Order)A->rg.order, S, cmin, cmax, nullptr);
+                for (uint32_t i = 0; i < sorted.size(); ++i) rank[sorted[i]] = i;
+                std::sort(sg[0].begin(), sg[0].end(),
+                          [&](const Grp& a, const Grp& b) { return rank[rows[a.first]] < rank[rows[b.first]]; });
             }
-            while (s < nseg) seg[s++] = rows.size();
-            seg[0] = 0;
-        }
-        sg.resize(nseg);
-        su.resize(nseg);
-        ok = parallel_for(nseg, [&](uint32_t s, uint32_t) {
-            Marks mk(ncols);
-            std::vector<uint32_t> U;
-            form_groups(M, rows.data() + seg[s], cube.empty() ? nullptr : cube.data() + seg[s], seg[s + 1] - seg[s], hr, mk, U,
-                        [&](size_t first, uint32_t cnt, const std::vector<uint32_t>& u) {
-                            sg[s].push_back({(uint32_t)(seg[s] + first), cnt, (uint32_t)u.size(), su[s].size()});
-                            su[s].insert(su[s].end(), u.begin(), u.end());
-                        });
-        });
-        if (!ok) throw std::bad_alloc();
+        } else {
+            const Strides S = find_strides(M, rows, cmin, cmax);
+            R.line = S.line;
+            R.plane = S.plane;
+            choose_order(M, rows, S, cmin, cmax, R.iw, es <= 2 ? 8 : 4, order, R.hr);
+            std::vector<uint8_t> cube;
+            if (!order_rows(M, rows, order, S, cmin, cmax, &cube)) order = ORDER_MATRIX;
+            const uint32_t hr = R.hr;
+
+            // groups, formed segment by segment (four segments per CTA, about equal entries)
+            const uint32_t nseg = std::max<uint32_t>(1, std::min<uint32_t>(4 * grid, (uint32_t)(rows.size() / 256)));
+            std::vector<size_t> seg(nseg + 1, rows.size());
+            {
+                uint64_t run = 0;
+                uint32_t s = 0;
+                for (size_t i = 0; i < rows.size(); ++i) {
+                    while (s < nseg && run * nseg >= (uint64_t)s * A->nnz) seg[s++] = i;
+                    run += rp[rows[i] + 1] - rp[rows[i]];
+                }
+                while (s < nseg) seg[s++] = rows.size();
+                seg[0] = 0;
+            }
+            sg.resize(nseg);
+            su.resize(nseg);
+            ok = parallel_for(nseg, [&](uint32_t s, uint32_t) {
+                Marks mk(ncols);
+                std::vector<uint32_t> U;
+                form_groups(M, rows.data() + seg[s], cube.empty() ? nullptr : cube.data() + seg[s], seg[s + 1] - seg[s], hr, mk, U,
+                            [&](size_t first, uint32_t cnt, const std::vector<uint32_t>& u) {
+                                sg[s].push_back({(uint32_t)(seg[s] + first), cnt, (uint32_t)u.size(), su[s].size()});
+                                su[s].insert(su[s].end(), u.begin(), u.end());
+                            });
+            });
+            if (!ok) throw std::bad_alloc();
         }
         const uint32_t hr = R.hr;
         // contiguous runs of groups of equal cost, one per CTA
@@ -907,8 +932,8 @@ bool build_row_groups(dose_matrix* A, RowGroups& R, bool keep, const uint32_t* r
             return false;
         }
         std::vector<std::vector<std::pair<const Grp*, const uint32_t*>>> cta(grid);
-        std::vector<std::vector<uint32_t>> tag(keep ? grid : 0);
-        if (keep) {
+        std::vector<std::vector<uint32_t>> tag(kept_deal ? grid : 0);
+        if (kept_deal) {
             for (uint32_t c = 0; c < grid; ++c)
                 for (uint32_t w = 0; w < R.keep_nw; ++w)
                     for (uint32_t d = KS.cta_begin[c]; d < KS.cta_begin[c + 1]; ++d) {
@@ -929,7 +954,7 @@ bool build_row_groups(dose_matrix* A, RowGroups& R, bool keep, const uint32_t* r
                 }
         }
         // small matrices: packets small enough that a warp gets several
-        const uint32_t pack = keep ? max_u : (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(cap, n_union / ((uint64_t)grid * 96)));
+        const uint32_t pack = kept_deal ? max_u : (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(cap, n_union / ((uint64_t)grid * 96)));
         std::vector<CtaOut> out(grid);
         struct Work {
             std::vector<uint32_t> pos, seen;
@@ -942,7 +967,8 @@ bool build_row_groups(dose_matrix* A, RowGroups& R, bool keep, const uint32_t* r
                 w.pos.assign(std::max(ncols, 1u), 0);
                 w.seen.assign(std::max(ncols, 1u), 0);
             }
-            write_cta(M, hr, R.iw, pack, max_u, rows.data(), cta[c], keep ? &tag[c] : nullptr, !forward_only, w.pos, w.seen, ++w.gen, out[c]);
+            write_cta(M, hr, R.iw, pack, max_u, rows.data(), cta[c], keep, kept_deal ? &tag[c] : nullptr,
+                      !forward_only, w.pos, w.seen, ++w.gen, out[c]);
         });
         if (!ok) throw std::bad_alloc();
 
@@ -1038,7 +1064,7 @@ bool build_row_groups(dose_matrix* A, RowGroups& R, bool keep, const uint32_t* r
         R.n_union = n_union;
         R.tile_u = tile_u;
         R.order = (uint32_t)order;
-        R.keep = keep;
+        R.keep = kept_deal;
         R.forward_only = forward_only;
         R.data_bytes = bytes;
         R.bytes = bytes + row_list.size() * 4 + dict.size() * 12 + (size_t)ncols * 32 + zr.size() * 8 + mask.size() * 4;

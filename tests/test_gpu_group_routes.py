@@ -124,3 +124,28 @@ def test_fused_pass_of_a_large_plan(fmt):
     A = dose.DoseMatrix.from_multibeam([(e.row_ptr, e.col, e.ncols, e.values, None) for e in encs], fmt=fmt)
     assert (A.info()["rg_order"], A.info()["rg_rows"]) == (CUBES, 8)
     _check(A, csr, oracle.encode(csr, OFMT[fmt]))
+
+
+@pytest.mark.parametrize("fmt", ["u16", "fp8", "f32"])
+def test_fused_pass_of_medium_beams(fmt):
+    """Between 100,000 and 200,000 rows with entries: the stored-row groups on the other
+    layout's deal (FP8: on their own)."""
+    csr = _route("planes")
+    assert 100000 < np.count_nonzero(csr.row_lengths()) < 200000
+    A, enc = make(csr, fmt)
+    _check(A, csr, enc)
+
+
+@pytest.mark.parametrize("fmt", ["bf16", "f32"])
+def test_fused_pass_of_a_medium_plan(fmt):
+    """100,000 to 400,000 rows with entries, unions of several packets; a second call
+    gives the same bits."""
+    beams, csr = _plan((72, 70, 50), (18, 12))
+    assert 100000 < np.count_nonzero(csr.row_lengths()) < 400000 and csr.row_lengths().max() > 320
+    encs = [oracle.encode(b, OFMT[fmt]) for b in beams]
+    A = dose.DoseMatrix.from_multibeam([(e.row_ptr, e.col, e.ncols, e.values, None) for e in encs], fmt=fmt)
+    _check(A, csr, oracle.encode(csr, OFMT[fmt]))
+    x, p, w = (_to(np.random.default_rng(k).uniform(0, 1, n).astype(np.float32))
+               for k, n in ((1, csr.ncols), (2, csr.nrows), (3, csr.nrows)))
+    for a, b in zip(A.fwd_adj_quadratic(x, p, w, want_d=True), A.fwd_adj_quadratic(x, p, w, want_d=True)):
+        assert torch.equal(a, b)
