@@ -949,6 +949,9 @@ static dose_status create_matrix(const dose_csr_desc* desc, unsigned flags, cons
                 return fail(e, "row-group schedule");
             }
         }
+        // a layout of the forward calls alone that none of them would take
+        const dose_matrix* self = A.get();
+        if (ok && A->rg.forward_only && !spmv_on_row_groups(self) && !rg_spmm_applies(&self, 1, nullptr)) free_row_groups(A->rg);
         if (A->adj_tuning.layout == 2 && !(ok && rg_active(A.get(), false))) {
             free_all(A.get());
             set_error("adj_layout = 2: the row-group layout does not apply" + (why.empty() ? std::string() : ": " + why));
@@ -1103,9 +1106,9 @@ dose_status dose_spmv_f64(const dose_matrix* A, const double* x, double* d, unsi
 namespace dose {
 // dose_spmv runs on the row-group layout unless the caller asked for CSR
 // (fwd_layout = 1), the handle sums long rows with compensation (a CSR path),
-// or the layout is missing or its ring does not fit beside the window of x.
+// or the layout is missing or too few warps fit beside the window of x.
 bool spmv_on_row_groups(const dose_matrix* A) {
-    return A->fwd.tuning.layout != 1 && !(A->flags & DOSE_CREATE_COMPENSATED) && rg_forward_warps(A, RG_DEAL_SPMV, nullptr, nullptr) > 0;
+    return A->fwd.tuning.layout != 1 && !(A->flags & DOSE_CREATE_COMPENSATED) && rg_spmv_applies(A);
 }
 
 dose_status adjoint_supported(const dose_matrix* A, bool quad, const float* const* vecs, int nvec) {

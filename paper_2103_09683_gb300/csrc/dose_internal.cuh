@@ -334,7 +334,9 @@ uint64_t rg_fused_bytes(const dose_matrix* A, bool with_d);
 // matrices A[0 .. count), and in how many launches.
 constexpr uint32_t kRgSpmmMaxPerLaunch = 32;
 bool rg_spmm_applies(const dose_matrix* const* A, int count, int* launches);
-// dose_spmv_f64 on the row-group layout (rg_spmm.cu).
+// dose_spmv and dose_spmv_f64 on the row-group layout (rg_spmm.cu): whether it is the
+// better form (fwd_layout = 2: whether it fits).
+bool rg_spmv_applies(const dose_matrix* A);
 bool rg_spmv64_applies(const dose_matrix* A);
 cudaError_t launch_rg_spmv64(const dose_matrix* A, const double* x, double* d, bool native, cudaStream_t s);
 // Whether dose_spmv takes the row-group form for this handle (dose_api.cu).

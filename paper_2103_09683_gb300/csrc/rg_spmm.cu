@@ -613,7 +613,27 @@ cudaError_t launch_rg_spmv(const dose_matrix* A, const float* x, float* d, cudaS
     });
 }
 
-bool rg_spmv64_applies(const dose_matrix* A) { return rg_forward_warps(A, RG_DEAL_F64, nullptr, nullptr) > 0; }
+// dose_spmv by default needs three warps beside the CTA's columns of x (51,000 of them):
+// 60,000 rows of 300 scattered entries take 95 us with five warps (46,800 columns) and
+// 203 us on CSR, so about 160 us with three and 240 with two.
+bool rg_spmv_applies(const dose_matrix* A) {
+    return rg_forward_warps(A, RG_DEAL_SPMV, nullptr, nullptr) >= (A->fwd.tuning.layout == 2 ? 1u : 3u);
+}
+
+// dose_spmv_f64 by default: the arithmetic bounds it, and row groups pay it for every
+// stored value, CSR for every entry (2.4 times as much, and a launch).  200 x 200 x 120
+// beam with some entries taken out, F16, stored values per entry 1.08 / 2.05 / 2.64 /
+// 3.06: 61 / 80 / 81 / 71 us against 112 / 89 / 75 / 49 on CSR; FP8 and F32 alike.  On
+// small matrices the launch decides (2e6 entries' worth).  Fewer than 14 warps beside
+// the columns of x (8 bytes each) cost about (warps + 2) / 16: 120,000 rows of 300
+// scattered entries, eight alike, with 14 / 9 / 6 / 4 / 3 warps 36 / 52 / 68 / 88 / 111
+// us, 83 to 95 on CSR.
+bool rg_spmv64_applies(const dose_matrix* A) {
+    const uint64_t nw = rg_forward_warps(A, RG_DEAL_F64, nullptr, nullptr);
+    if (!nw || A->fwd.tuning.layout == 2) return nw > 0;
+    const uint64_t stored = A->rg.n_union * A->rg.hr;
+    return 16 * stored <= (std::min<uint64_t>(nw, 14) + 2) * (A->nnz * 12ull / 5 + 2000000);
+}
 
 cudaError_t launch_rg_spmv64(const dose_matrix* A, const double* x, double* d, bool native, cudaStream_t s) {
     FwdParams p;
