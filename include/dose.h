@@ -163,24 +163,31 @@ typedef struct {
     uint32_t adj_layout;
     uint32_t rg_tile_union;     /* row groups: union columns a warp copies at a time (256..8192, at least the
                                    longest row where that is at most 4096; at most 320 are used).  Packets are
-                                   cut at create; a later value is checked and reported only.  Where the
-                                   fused pass keeps the stored-row order (see rg_groups in dose_info), also
-                                   the union columns of one stage of that order.  Default by format (2048 to
-                                   6816), at least the longest row. */
-    uint32_t rg_tile_rows;      /* row groups: rows a stage of the stored-row order spans, at create (256..8192;
+                                   cut at create; a later value is checked and reported only.  Also the
+                                   union columns of one stage of the kept order (see rg_warps).  Default by
+                                   format (2048 to 6816), at least the longest row. */
+    uint32_t rg_tile_rows;      /* row groups: rows that a stage of the kept order spans, at create (256..8192;
                                    default 512); a packet holds at most 64 rows */
     uint32_t rg_stages;         /* row groups: packets in flight per warp of the adjoint and fused passes
                                    (2..8; at most 4 are used; default 2) */
-    uint32_t rg_warps;          /* row groups: worker warps of those passes (1..15; 0 = as many as fit) */
+    uint32_t rg_warps;          /* row groups: worker warps of those passes (1..15; 0 = as many as fit).  The
+                                   fused pass of matrices of fewer than 100,000 rows with entries (FP8:
+                                   200,000, plans 400,000) deals its groups to warps in a kept order, cut at
+                                   create by rg_tile_union, rg_tile_rows, rg_stages and rg_warps: given there
+                                   they set the order in which the gradient is added, given later rg_warps
+                                   folds the warps cut at create onto fewer */
     uint32_t rg_l2_prefetch;    /* row groups: checked and reported; the passes need no L2 prefetch */
     uint32_t fwd_layout;        /* layout dose_spmv runs on: 0 = row groups where the handle has them
-                                   (and not DOSE_CREATE_COMPENSATED, whose long-row sums run on CSR),
-                                   else CSR (default); 1 = CSR; 2 = row groups (create and
+                                   (and not DOSE_CREATE_COMPENSATED, whose long-row sums run on CSR)
+                                   and three warps fit beside a CTA's columns of x (up to about 51,000
+                                   of them), else CSR (default); 1 = CSR; 2 = row groups (create and
                                    dose_set_tuning fail if dose_spmv cannot take them).  On row groups
                                    a row's terms are added in its group's union order (see adj_layout),
                                    so the last bits may differ from the CSR form's.  dose_spmv_f64 follows
-                                   dose_spmv, except that DOSE_SPMV_F64_NATIVE takes row groups only with
-                                   fwd_layout = 2 (FP64 FMAs bound it, and CSR stores fewer values). */
+                                   dose_spmv where the groups store few zeros (up to about 1.4 zeros per
+                                   entry, fewer where few warps fit), and DOSE_SPMV_F64_NATIVE takes row
+                                   groups only with fwd_layout = 2 (FP64 FMAs bound it, and CSR stores
+                                   fewer values). */
 } dose_tuning;
 
 typedef struct {
@@ -261,8 +268,10 @@ dose_status dose_spmv(const dose_matrix* A, const float* x, float* d, void* stre
  * product is formed to ~2^-47 relative with FMAs, and sums are double-float pairs
  * (TwoSum); row results are rounded once to FP64.  A row of n entries then has
  * |d_i - sum_k a_ik x_k| <= (2^-45 + g(m)^2) sum_k |a_ik x_k| + 2^-53 |d_i|, where
- * m <= n is the most terms any one accumulator of the row adds (a handful on the
- * default schedule) and g(m) = m 2^-24 / (1 - m 2^-24).  DOSE_SPMV_F64_NATIVE
+ * m <= n is the most terms any one accumulator of the row adds (a handful on the CSR
+ * arrays' default schedule; on row groups one for every 32 columns of the row's group,
+ * at most 128, and at most 2048 where rows have more than 4096 entries) and
+ * g(m) = m 2^-24 / (1 - m 2^-24).  DOSE_SPMV_F64_NATIVE
  * accumulates with FP64 FMAs: |error| <= (n + 2) 2^-53 sum_k |a_ik x_k|.
  * On the CSR arrays it uses a handle-owned scratch copy of x (ncols + 1 doubles)
  * and two launches on `stream`, on row groups one launch; the same-stream rule for

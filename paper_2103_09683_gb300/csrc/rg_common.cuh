@@ -66,11 +66,11 @@ inline RgView rg_view(const dose_matrix* A, int which) {
 #ifdef __CUDACC__
 
 namespace dev {
-// All bulk stores of this thread done (source read and data written).
 __device__ __forceinline__ void bulk_s2g(void* dst, const void* src, uint32_t bytes) {
     asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_u32(src)), "r"(bytes)
                  : "memory");
 }
+// All bulk stores of this thread done (source read and data written).
 __device__ __forceinline__ void bulk_store_wait() {
     asm volatile("cp.async.bulk.commit_group;\n\tcp.async.bulk.wait_group 0;" ::: "memory");
 }

@@ -379,9 +379,9 @@ __global__ void __launch_bounds__((kRgMaxWarps + kRgRowWarps) * 32, 1) rg_kernel
     if (p.chain & RG_CHAIN_PREV) rg_wait_previous();
 }
 
-// Second kernel of the row-group passes: column block cb: g_j = s * (sum of the partials of the CTAs that see column j, in CTA
-// order), and the optional projected-gradient step on x; block 0 also writes f =
-// the CTAs' objective partials, added in one fixed order.
+// Second kernel of the row-group passes: g_j = s * (sum of the partials of the CTAs
+// that see column j, in CTA order), and the optional projected-gradient step on x;
+// block 0 also writes f = the CTAs' objective partials, added in one fixed order.
 struct RgFin {
     const float* g_part;
     const uint32_t* col_ptr;  // where column j's partials lie in g_part (CTA order)
