@@ -74,12 +74,12 @@ cudaError_t rg_upload(void** dst, const void* src, size_t bytes, size_t alloc_by
     return e;
 }
 
-// fn(i, thread) for i < n on several threads; false if a thread could not get
-// memory (no exception leaves a thread).
+// fn(i, thread) for i < n on several threads (at most `most`); false if a thread could
+// not get memory (no exception leaves a thread).
 constexpr uint32_t kMaxThreads = 32;
 template <class F>
-bool parallel_for(uint32_t n, F fn) {
-    const uint32_t nt = std::max(1u, std::min({n, kMaxThreads, std::thread::hardware_concurrency()}));
+bool parallel_for(uint32_t n, F fn, uint32_t most = kMaxThreads) {
+    const uint32_t nt = std::max(1u, std::min({n, most, kMaxThreads, std::thread::hardware_concurrency()}));
     std::atomic<uint32_t> next{0};
     std::atomic<bool> ok{true};
     auto work = [&](uint32_t thread) {
@@ -313,58 +313,67 @@ bool order_rows(const Csr& A, std::vector<uint32_t>& rows, Order o, const Stride
 void choose_order(const Csr& A, const std::vector<uint32_t>& rows, const Strides& S, const uint32_t* cmin,
                   const uint32_t* cmax, uint32_t iw, uint32_t hr_hi, Order& order, uint32_t& hr) {
     constexpr uint32_t kSamples = 48;
-    std::vector<uint32_t> U, set;
-    Marks mk(A.ncols);
     const size_t n = rows.size();
+    std::vector<Order> orders{ORDER_MATRIX};
+    if (S.plane) orders.push_back(ORDER_PLANES);
+    if (S.line) orders.push_back(ORDER_CUBES);
+    std::vector<uint32_t> by_col;
+    if (!S.plane) {  // (else the grid orders know more)
+        orders.push_back(ORDER_COLUMNS);
+        by_col = rows;
+        order_rows(A, by_col, ORDER_COLUMNS, S, cmin, cmax, nullptr);
+    }
+    // on several threads where rows have thousands of entries (1.05e8 entries in 1.35e5
+    // rows: 48 -> 8 ms on eight); a millisecond of work otherwise, less than the threads
+    const bool threads = A.rp[A.nrows] / std::max<size_t>(n, 1) >= 512;
+    std::vector<Estimate> est(orders.size() * kSamples * 2);  // of 4 and of 8 rows
+    std::vector<std::unique_ptr<Marks>> marks(kMaxThreads);
+    const bool ok = parallel_for((uint32_t)orders.size() * kSamples, [&](uint32_t task, uint32_t thread) {
+        if (!marks[thread]) marks[thread].reset(new Marks(A.ncols));
+        Marks& mk = *marks[thread];
+        const Order o = orders[task / kSamples];
+        const size_t i = (size_t)((uint64_t)n * (2 * (task % kSamples) + 1) / (2 * kSamples));
+        std::vector<uint32_t> U, set;
+        if (o == ORDER_MATRIX || o == ORDER_COLUMNS) {
+            const std::vector<uint32_t>& src = o == ORDER_MATRIX ? rows : by_col;
+            for (size_t k = i; k < std::min(n, i + 64); ++k) set.push_back(src[k]);
+        } else if (o == ORDER_PLANES) {
+            const uint64_t z0 = rows[i] / S.plane, zb = z0 > 128 ? z0 - 128 : 0;
+            for (uint64_t z = zb; z < zb + 256; ++z) {
+                const uint64_t r = z * S.plane + rows[i] % S.plane;
+                if (r >= A.nrows) break;
+                if (A.rp[r + 1] > A.rp[r]) set.push_back((uint32_t)r);
+            }
+        } else {
+            const uint64_t z = rows[i] / S.plane / 2 * 2, q = rows[i] % S.plane, y = q / S.line / 2 * 2, x = q % S.line / 8 * 8,
+                           ny = S.plane / S.line;
+            for (uint64_t c = 0; c < 4; ++c)
+                for (uint64_t k = 0; k < 8; ++k) {
+                    const uint64_t zz = z + (k >> 2), yy = y + ((k >> 1) & 1), xx = x + 2 * c + (k & 1);
+                    const uint64_t r = zz * S.plane + yy * S.line + xx;
+                    if (yy < ny && xx < S.line && r < A.nrows && A.rp[r + 1] > A.rp[r]) set.push_back((uint32_t)r);
+                }
+        }
+        for (uint32_t h : {4u, 8u})
+            if (h <= hr_hi) estimate_add(A, set, h, iw, mk, U, est[2 * task + h / 8]);
+    }, threads ? kMaxThreads : 1);
+    if (!ok) throw std::bad_alloc();
     double best = 1e30;
     order = ORDER_MATRIX;
     hr = hr_hi;
-    std::vector<uint32_t> by_col;
-    for (int o = ORDER_MATRIX; o <= ORDER_COLUMNS; ++o) {
-        if (o == ORDER_PLANES && !S.plane) continue;
-        if (o == ORDER_CUBES && !S.line) continue;
-        if (o == ORDER_COLUMNS) {
-            if (S.plane) continue;  // the grid orders know more
-            by_col = rows;
-            order_rows(A, by_col, ORDER_COLUMNS, S, cmin, cmax, nullptr);
-        }
+    for (size_t j = 0; j < orders.size(); ++j)
         for (uint32_t h : {4u, 8u}) {
-            if (h > hr_hi) continue;
             Estimate e;
             for (uint32_t s = 0; s < kSamples; ++s) {
-                const size_t i = (size_t)((uint64_t)n * (2 * s + 1) / (2 * kSamples));
-                set.clear();
-                if (o == ORDER_MATRIX || o == ORDER_COLUMNS) {
-                    const std::vector<uint32_t>& src = o == ORDER_MATRIX ? rows : by_col;
-                    for (size_t k = i; k < std::min(n, i + 64); ++k) set.push_back(src[k]);
-                    estimate_add(A, set, h, iw, mk, U, e);
-                } else if (o == ORDER_PLANES) {
-                    const uint64_t z0 = rows[i] / S.plane, zb = z0 > 128 ? z0 - 128 : 0;
-                    for (uint64_t z = zb; z < zb + 256; ++z) {
-                        const uint64_t r = z * S.plane + rows[i] % S.plane;
-                        if (r >= A.nrows) break;
-                        if (A.rp[r + 1] > A.rp[r]) set.push_back((uint32_t)r);
-                    }
-                    estimate_add(A, set, h, iw, mk, U, e);
-                } else {
-                    const uint64_t z = rows[i] / S.plane / 2 * 2, q = rows[i] % S.plane, y = q / S.line / 2 * 2,
-                                   x = q % S.line / 8 * 8, ny = S.plane / S.line;
-                    for (uint64_t c = 0; c < 4; ++c)
-                        for (uint64_t k = 0; k < 8; ++k) {
-                            const uint64_t zz = z + (k >> 2), yy = y + ((k >> 1) & 1), xx = x + 2 * c + (k & 1);
-                            const uint64_t r = zz * S.plane + yy * S.line + xx;
-                            if (yy < ny && xx < S.line && r < A.nrows && A.rp[r + 1] > A.rp[r]) set.push_back((uint32_t)r);
-                        }
-                    estimate_add(A, set, h, iw, mk, U, e);
-                }
+                e.bytes += est[2 * (j * kSamples + s) + h / 8].bytes;
+                e.entries += est[2 * (j * kSamples + s) + h / 8].entries;
             }
-            if (e.per_entry() < 0.98 * best) {
+            if (h <= hr_hi && e.per_entry() < 0.98 * best) {
                 best = e.per_entry();
-                order = (Order)o;
+                order = orders[j];
                 hr = h;
             }
         }
-    }
 }
 
 struct Grp {
