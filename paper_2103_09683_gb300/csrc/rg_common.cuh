@@ -111,10 +111,7 @@ struct RgDict {
         decltype(get(0u)) v[4];
 #pragma unroll
         for (uint32_t k = 0; k < 2; ++k)
-            if (t + k * nt < nc) v[k] = get(c[k]);
-#pragma unroll
-        for (uint32_t k = 0; k < 2; ++k)
-            if (t + k * nt < nc) put(t + k * nt, v[k]);
+            if (t + k * nt < nc) put(t + k * nt, get(c[k]));
         for (uint32_t j = t + 2 * nt; j < nc; j += 4 * nt) {
             uint32_t q[4];
 #pragma unroll
